@@ -121,10 +121,10 @@ typedef struct {
                           kernel, 512 for the per-thread cp.async prefetch
                           kernel, 4096 for the plain kernel on a persistent
                           grid of contiguous site ranges, 8192 for the
-                          tensor-core stencil (mma.sync): in the F64 form
-                          double-float values split into bf16 slices with
-                          exact products (N = 16 or 32 with a workspace set;
-                          the cp.async kernel otherwise), in the FP16 and
+                          tensor-core stencil (mma.sync): double-float and
+                          FP64 as exact products of 8-bit digits (N >= 2 with
+                          a workspace set; the cp.async or the plain kernel
+                          otherwise), in the FP16 and
                           bfloat16 forms the stored values themselves (N = 16
                           or 32 with full links; the plain kernel
                           otherwise).  Other values: BLOCKCG_ERR_ARG */

@@ -80,6 +80,7 @@ struct blockcg_ctx {
 namespace {
 
 const size_t ALIGN = 256;
+const size_t FX_CTL_BYTES = 1024;  // a multiple of ALIGN
 inline size_t up(size_t x) { return (x + ALIGN - 1) / ALIGN * ALIGN; }
 
 enum MatId { M_H = 0, M_G, M_C, M_CPREV, M_BETA, M_BC, M_SINV, M_SH, M_CINV, M_SHRU, M_K, M_RINV, M_COUNT };
@@ -111,9 +112,10 @@ Ws carve(const blockcg_ctx* h, int N, char* base) {
     off += up(bytes);
     return p;
   };
-  // first: the tensor-core stencil's column maxima, at an offset that does
-  // not depend on N (Geom::tc_colmax points here once the workspace is set)
-  take(64 * sizeof(unsigned));
+  // first: the digit stencil's control words and input digits, at offsets
+  // that do not depend on N (Geom::fx_ctl and fx_dig, set with the workspace)
+  take(FX_CTL_BYTES);
+  take(fx_digit_bytes(h->g, N));
   size_t nel = (size_t)h->g.Vh * N * 3;
   size_t fb = nel * elem_bytes(h->fine), rb = nel * elem_bytes(h->ru),
          sb = nel * elem_bytes(h->sloppy);
@@ -347,6 +349,22 @@ int recon_flag(const blockcg_ctx* h, FieldKind k) {
              : 0;
 }
 
+// FP64 blocks of N >= 4: the digit stencil only.  The CUDA-core kernels are
+// bound by the FP64 rate (one half at 32^4, N = 16: 7.8 ms against 1.6 with the
+// digits of its input; 8^4, N = 4: 45 against 21 us); at N = 2 and 16^4 they
+// are still the faster ones (84 against 96 us).  In the forms that use FP64 in
+// the reliable updates alone, whose launches are enqueued every iteration and
+// mostly gated off, small problems keep the CUDA-core kernels too: the digit
+// stencil is three launches more (12.8.10.14, N = 5: 29.0 against 32.1 ms a
+// solve; 16^4, N = 8: 147 against 143).
+bool fx_allowed(const blockcg_ctx* h, FieldKind k, int N) {
+  return dslash_fx_supported(h->g, N) &&
+         (k != FK_F64 || h->sloppy == FK_F64 || (long long)h->g.Vh * N >= 1 << 18);
+}
+bool fx_only(const blockcg_ctx* h, FieldKind k, int N) {
+  return k == FK_F64 && N >= 4 && fx_allowed(h, k, N);
+}
+
 // Autotuned stencil choice for (kind, N), cached.  Each candidate is timed
 // over 3 launches of out = D in; with out2 the candidate is timed on the pair
 // the normal operator runs (out = D_oe in, then out2 = m^2 in - D_eo out), so
@@ -379,10 +397,10 @@ int stencil_R(blockcg_ctx* h, FieldKind k, int N, const void* links, const void*
                          1 | DSLASH_TC};
   for (int R : cands) {
     if ((R & 0xff) > 1 && (R & 0xff) > N) continue;
-    // the tensor-core stencil: double-float, FP16 and bfloat16 with N = 16 or
-    // 32 and full links only
+    // the tensor-core stencil: double-float and FP64, and FP16 and bfloat16
+    // with N = 16 or 32 and full links
     if ((R & DSLASH_TC) &&
-        (rf || !((k == FK_DF && dslash_tc_supported(h->g, N)) ||
+        (rf || !(((k == FK_DF || k == FK_F64) && fx_allowed(h, k, N)) ||
                  ((k == FK_H16 || k == FK_BF16) && dslash_tc16_supported(N)))))
       continue;
     if (rf) {  // two-row links: the plain kernel only
@@ -395,12 +413,14 @@ int stencil_R(blockcg_ctx* h, FieldKind k, int N, const void* links, const void*
     // in repeated 32^4 N = 16 measurements, while the cp.async kernel ran as
     // timed.
     if (k == FK_DF && N >= 2 && !(R & (DSLASH_ASYNC | DSLASH_TC))) continue;
+    if (fx_only(h, k, N) && !(R & DSLASH_TC)) continue;
     const double m2 = h->mass * h->mass;
     auto run = [&]() {
-      cudaError_t e = dslash(k, R, EPI_NONE, links, in, out, nullptr, nullptr, 0.0, h->g, 1, N, g0,
-                             h->stream);
+      cudaError_t e = dslash(k, out2 ? R | DSLASH_FIRST : R, EPI_NONE, links, in, out, nullptr,
+                             nullptr, 0.0, h->g, 1, N, g0, h->stream);
       if (e == cudaSuccess && out2)
-        e = dslash(k, R, EPI_NORMAL, links, out, out2, in, nullptr, m2, h->g, 0, N, g0, h->stream);
+        e = dslash(k, R | DSLASH_SECOND, EPI_NORMAL, links, out, out2, in, nullptr, m2, h->g, 0, N,
+                   g0, h->stream);
       return e;
     };
     if (run() != cudaSuccess) {
@@ -549,7 +569,8 @@ int cached_R(const blockcg_ctx* h, FieldKind k, int N) {
   const int rf = recon_flag(h, k);
   if (h->p.dslash_variant) return h->p.dslash_variant | rf;
   auto it = h->tuned_R.find((int)k * 128 + N);
-  return it != h->tuned_R.end() ? it->second : (tile_R(N) | rf);
+  if (it != h->tuned_R.end()) return it->second;
+  return fx_only(h, k, N) ? (1 | DSLASH_TC) : (tile_R(N) | rf);
 }
 
 blockcg_status check_ready(blockcg_ctx* h, int N) {
@@ -570,8 +591,10 @@ blockcg_status apply_A_internal(blockcg_ctx* h, FieldKind k, const void* links, 
                                 void* tmp_odd, void* out, int N, Gate gate) {
   int R = stencil_R(h, k, N, links, in, tmp_odd, out);
   double m2 = h->mass * h->mass;
-  KL(dslash(k, R, EPI_NONE, links, in, tmp_odd, nullptr, nullptr, 0.0, h->g, 1, N, gate, h->stream));
-  KL(dslash(k, R, EPI_NORMAL, links, tmp_odd, out, in, nullptr, m2, h->g, 0, N, gate, h->stream));
+  KL(dslash(k, R | DSLASH_FIRST, EPI_NONE, links, in, tmp_odd, nullptr, nullptr, 0.0, h->g, 1, N,
+            gate, h->stream));
+  KL(dslash(k, R | DSLASH_SECOND, EPI_NORMAL, links, tmp_odd, out, in, nullptr, m2, h->g, 0, N, gate,
+            h->stream));
   return BLOCKCG_OK;
 }
 
@@ -610,8 +633,9 @@ blockcg_status restart_residual(blockcg_ctx* h, const Ws& w, int N, double tol, 
   cudaStream_t s = h->stream;
   if (!skip_acc) TL(TC_STREAM, accumulate(h->fine, h->upd, w.Y, w.X, nel, gate, s));
   if (cheap) TL(TC_STREAM, convert_field(h->fine, rk, w.Y, Yk, nel, nullptr, gate, s));
-  SL(1, dslash(rk, R, EPI_NONE, links, Yk, w.Tf, nullptr, nullptr, 0.0, h->g, 1, N, gate, s));
-  SL(1, dslash(rk, R, EPI_RESIDUAL, links, w.Tf, Rk, Yk, Bk, m2, h->g, 0, N, gate, s));
+  SL(1, dslash(rk, R | DSLASH_FIRST, EPI_NONE, links, Yk, w.Tf, nullptr, nullptr, 0.0, h->g, 1, N,
+               gate, s));
+  SL(1, dslash(rk, R | DSLASH_SECOND, EPI_RESIDUAL, links, w.Tf, Rk, Yk, Bk, m2, h->g, 0, N, gate, s));
   TL(TC_GRAM, gram_partials(rk, Rk, Rk, N, h->g.Vh, 1, w.partials, w.nblocks, gate, s));
   TL(TC_GRAM, gram_reduce(w.partials, w.nblocks, N, 1, mat(w, M_G, N), gate, s));
   TL(TC_DENSE, dense_restart(mat(w, M_G, N), mat(w, M_C, N), mat(w, M_CPREV, N), mat(w, M_CINV, N),
@@ -663,8 +687,10 @@ blockcg_status verify_fp64(blockcg_ctx* h, const Ws& w, int N, double tol) {
   const double m2 = h->mass * h->mass;
   cudaStream_t s = h->stream;
   Gate g0{nullptr, GATE_ALWAYS};
-  SL(1, dslash(FK_F64, R, EPI_NONE, h->links_fine, w.Y, w.Tf, nullptr, nullptr, 0.0, h->g, 1, N, g0, s));
-  SL(1, dslash(FK_F64, R, EPI_RESIDUAL, h->links_fine, w.Tf, w.R, w.Y, w.B, m2, h->g, 0, N, g0, s));
+  SL(1, dslash(FK_F64, R | DSLASH_FIRST, EPI_NONE, h->links_fine, w.Y, w.Tf, nullptr, nullptr, 0.0,
+               h->g, 1, N, g0, s));
+  SL(1, dslash(FK_F64, R | DSLASH_SECOND, EPI_RESIDUAL, h->links_fine, w.Tf, w.R, w.Y, w.B, m2, h->g,
+               0, N, g0, s));
   TL(TC_GRAM, gram_partials(FK_F64, w.R, w.R, N, h->g.Vh, 1, w.partials, w.nblocks, g0, s));
   TL(TC_GRAM, gram_reduce(w.partials, w.nblocks, N, 1, mat(w, M_K, N), g0, s));
   TL(TC_DENSE, dense_verify(mat(w, M_K, N), w.bnorm, w.tres, tol, N, w.st, s));
@@ -678,8 +704,10 @@ blockcg_status iterate_block(blockcg_ctx* h, const Ws& w, int N, double tol) {
   double m2 = h->mass * h->mass;
   cudaStream_t s = h->stream;
   FieldKind k = h->sloppy;
-  SL(0, dslash(k, R, EPI_NONE, h->links_sloppy, w.P, w.Ts, nullptr, nullptr, 0.0, h->g, 1, N, ga, s));
-  SL(0, dslash(k, R, EPI_NORMAL, h->links_sloppy, w.Ts, w.AP, w.P, nullptr, m2, h->g, 0, N, ga, s));
+  SL(0, dslash(k, R | DSLASH_FIRST, EPI_NONE, h->links_sloppy, w.P, w.Ts, nullptr, nullptr, 0.0, h->g,
+               1, N, ga, s));
+  SL(0, dslash(k, R | DSLASH_SECOND, EPI_NORMAL, h->links_sloppy, w.Ts, w.AP, w.P, nullptr, m2, h->g,
+               0, N, ga, s));
   const BlasTiles bt = cached_tiles(h, k, N);
   TL(TC_GRAM, gram_partials(k, w.P, w.AP, N, h->g.Vh, 1, w.partials, w.nblocks, ga, s, bt.gram));
   TL(TC_GRAM, gram_reduce(w.partials, w.nblocks, N, 1, mat(w, M_H, N), ga, s));
@@ -872,7 +900,9 @@ blockcg_status blockcg_create(blockcg_t* out, const int dims[4], double mass,
   h->g.antiperiodic = prm.antiperiodic_t ? 1 : 0;
   h->g.inv_c[0] = h->g.inv_c[1] = 0.f;
   h->g.wait_ns = (unsigned long long)prm.wait_limit_ns;
-  h->g.tc_colmax = nullptr;
+  h->g.fx_ctl = nullptr;
+  h->g.fx_dig = nullptr;
+  h->g.fx_links = nullptr;
   h->mass = mass;
   h->p = prm;
   h->stream = (cudaStream_t)stream;
@@ -917,6 +947,7 @@ size_t blockcg_gauge_bytes(blockcg_t h) {
   size_t b = up(links_bytes(h->fine, h->g));
   if (h->sloppy != h->fine) b += up(links_bytes(h->sloppy, h->g, h->p.link_recon));
   if (h->ru != h->fine && h->ru != h->sloppy) b += up(links_bytes(h->ru, h->g));
+  b += up(fx_links_bytes(h->g));
   if (h->p.link_recon) b += ALIGN;  // scratch of the link check
   return b;
 }
@@ -951,7 +982,7 @@ blockcg_status blockcg_load_gauge(blockcg_t h, const void* fat, const void* lng,
   h->gauge = storage;
   h->gauge_bytes = storage_bytes;
   // [FP64 links][iteration links, if another kind][reliable-update links, if
-  // a third kind]
+  // a third kind][the digit stencil's links]
   char* next = (char*)storage + up(links_bytes(h->fine, h->g));
   h->links_fine = storage;
   h->links_sloppy = storage;
@@ -968,6 +999,9 @@ blockcg_status blockcg_load_gauge(blockcg_t h, const void* fat, const void* lng,
   if (h->links_ru != h->links_fine && h->links_ru != h->links_sloppy)
     CK(pack_links(h->ru, (const double2*)fat, (const double2*)lng, h->links_ru, h->g,
                   h->p.antiperiodic_t, 0, h->stream));
+  if (h->ru != h->fine && h->ru != h->sloppy) next += up(links_bytes(h->ru, h->g));
+  CK(fx_pack_links(h->links_fine, next, h->g, h->stream));
+  h->g.fx_links = next;
   h->gauge_loaded = true;
   return BLOCKCG_OK;
 }
@@ -983,7 +1017,8 @@ blockcg_status blockcg_set_workspace(blockcg_t h, void* ws, size_t bytes) {
   if (((uintptr_t)ws) % 16) return fail(h, BLOCKCG_ERR_ARG, "workspace not 16-byte aligned");
   h->ws = (char*)ws;
   h->ws_bytes = bytes;
-  h->g.tc_colmax = (unsigned*)ws;  // the first region of carve()
+  h->g.fx_ctl = (unsigned*)ws;  // the first regions of carve()
+  h->g.fx_dig = (char*)ws + FX_CTL_BYTES;
   return BLOCKCG_OK;
 }
 

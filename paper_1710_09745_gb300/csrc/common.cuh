@@ -354,9 +354,12 @@ struct Geom {
   float inv_c[2];
   // bounded device waits (bulk-copy stencil) give up after this many ns
   unsigned long long wait_ns;
-  // the tensor-core double-float stencil's per-column maxima (64 words of the
-  // handle's workspace; null until a workspace is set)
-  unsigned* tc_colmax;
+  // the digit stencil (stencil_fx.cuh): control words and the input's digits
+  // in the handle's workspace (null until one is set), packed links in the
+  // gauge storage (null until a field is loaded)
+  unsigned* fx_ctl;
+  void* fx_dig;
+  const void* fx_links;
 };
 
 // coordinates of the site with checkerboard index cb on parity p

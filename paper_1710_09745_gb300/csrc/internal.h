@@ -86,19 +86,32 @@ static constexpr int DSLASH_RECON = 0x400;
 // R | DSLASH_BLOCKED: the plain kernel on a persistent grid whose blocks each
 // walk one contiguous range of sites (cache reuse of neighbours in L1)
 static constexpr int DSLASH_BLOCKED = 0x1000;
-// R | DSLASH_TC: the tensor-core stencil: double-float as split products
-// (stencil_tc.cu; N = 16 or 32 with a workspace set, the cp.async kernel
-// otherwise), FP16 / bfloat16 on the stored values (stencil_tc16.cu; N = 16
-// or 32 with full links, the plain kernel otherwise)
+// R | DSLASH_TC: the tensor-core stencil: double-float and FP64 as exact
+// digit products (stencil_fx.cuh; N >= 2 with a workspace set, the cp.async
+// or the plain kernel otherwise), FP16 / bfloat16 on the stored values
+// (stencil_tc16.cu; N = 16 or 32 with full links, the plain kernel otherwise)
 static constexpr int DSLASH_TC = 0x2000;
-bool dslash_tc_supported(const Geom& g, int N);
+// the two halves of an operator application, out2 = ... D (out = D in): the
+// first half keeps its output's column maxima for the second (digit stencil;
+// the other kernels ignore both flags)
+static constexpr int DSLASH_FIRST = 0x4000;
+static constexpr int DSLASH_SECOND = 0x8000;
+bool dslash_fx_supported(const Geom& g, int N);
+size_t fx_links_bytes(const Geom& g);
+size_t fx_digit_bytes(const Geom& g, int N);
+// the digit stencil's links from the packed FP64 ones
+cudaError_t fx_pack_links(const void* links_f64, void* storage, const Geom& g, cudaStream_t s);
 bool dslash_tc16_supported(int N);
 cudaError_t dslash_tc16(FieldKind k, int epi, const void* links, const void* in, void* out,
                         const void* c1, const void* c2, double m2, const Geom& g, int out_parity,
                         int N, Gate gate, cudaStream_t s);
-cudaError_t dslash_df_tc(int epi, const void* links, const void* in, void* out, const void* c1,
-                         const void* c2, double m2, const Geom& g, int out_parity, int N,
-                         Gate gate, cudaStream_t s);
+// flags: DSLASH_FIRST, DSLASH_SECOND
+cudaError_t dslash_fx_df(int flags, int epi, const void* links, const void* in, void* out,
+                         const void* c1, const void* c2, double m2, const Geom& g, int out_parity,
+                         int N, Gate gate, cudaStream_t s);
+cudaError_t dslash_fx_f64(int flags, int epi, const void* links, const void* in, void* out,
+                          const void* c1, const void* c2, double m2, const Geom& g, int out_parity,
+                          int N, Gate gate, cudaStream_t s);
 cudaError_t dslash(FieldKind k, int R, int epi, const void* links, const void* in, void* out,
                    const void* c1, const void* c2, double m2, const Geom& g, int out_parity,
                    int N, Gate gate, cudaStream_t s);

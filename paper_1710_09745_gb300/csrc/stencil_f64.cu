@@ -5,6 +5,8 @@
 namespace bcg {
 
 BCG_DSLASH_KIND_DECL(dslash_f64) {
+  if ((R & DSLASH_TC) && dslash_fx_supported(g, N))
+    return dslash_fx_f64(R, epi, links, in, out, c1, c2, m2, g, out_parity, N, gate, s);
   return dslash_kind<StoreF64>(R, epi, links, in, out, c1, c2, m2, g, out_parity, N, gate, s);
 }
 
