@@ -405,7 +405,7 @@ typedef struct blockcg_batch* blockcg_batch_t;
 #define BLOCKCG_BATCH_MAX 4096
 #define BLOCKCG_BATCH_GRAPH 1 /* flags bit: replay a captured CUDA graph */
 /* flags bits 8..15: iterations per device-loop trip with BLOCKCG_BATCH_GRAPH
- * (0: min(check_every, 4)) */
+ * (0: chosen from the problem's size; at most 16) */
 #define BLOCKCG_BATCH_TRIP_SHIFT 8
 
 typedef struct {

@@ -425,7 +425,7 @@ struct SolverStatus {
   int iters;           // iterations performed
   int reliable_updates;
   int stopped;         // 1: max_iter iterations done; the gated kernels stop
-  int trips;           // device-side loop trips (batched solves)
+  int trips;           // iterations run by a device-side loop
   double res_max;      // max relative iterated residual after the last iteration
   double res_at_ru;    // max relative residual at the last reliable update
   double true_res_max; // max relative true residual at the last check

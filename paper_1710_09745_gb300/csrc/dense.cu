@@ -167,18 +167,30 @@ __global__ void __launch_bounds__(DENSE_THREADS)
     k_dense_qr_step(const double2* __restrict__ G, double2* __restrict__ C,
                     double2* __restrict__ C_prev, double2* __restrict__ Sinv,
                     double2* __restrict__ SH, const double* __restrict__ bnorm, QrStepParams p,
-                    int N, SolverStatus* st, Gate gate) {
+                    int N, SolverStatus* st, Gate gate, LoopCtl ctl) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int flag;
   __shared__ double resv[64];
-  if (gate_closed(gate)) return;
+  if (gate_closed(gate)) {  // converged, failed or stopped: the loop ends
+    if (ctl.on && threadIdx.x == 0) {
+      cudaGraphSetConditional(ctl.update, 0);
+      cudaGraphSetConditional(ctl.loop, 0);
+    }
+    return;
+  }
   double2* A = reinterpret_cast<double2*>(smem_raw);
   double2* Li = A + N * N;
   double2* Cs = Li + N * N;
   load_mat(A, G, N);
   int f = chol_lower(A, N, &flag);
   if (f) {
-    if (threadIdx.x == 0) st->error = f;
+    if (threadIdx.x == 0) {
+      st->error = f;
+      if (ctl.on) {
+        cudaGraphSetConditional(ctl.update, 0);
+        cudaGraphSetConditional(ctl.loop, 0);
+      }
+    }
     return;
   }
   tri_inv_lower(A, Li, N);
@@ -225,16 +237,22 @@ __global__ void __launch_bounds__(DENSE_THREADS)
     else if (rmax > RU_GROWTH * st->res_at_ru) ru = 1;
     st->ru_pending = ru;
     // the iteration budget is spent: later chunks of gated launches do nothing
-    if (p.max_iter > 0 && it >= p.max_iter) st->stopped = 1;
+    const bool stop = p.max_iter > 0 && it >= p.max_iter;
+    if (stop) st->stopped = 1;
+    if (ctl.on) {
+      st->trips += 1;
+      cudaGraphSetConditional(ctl.update, ru && !stop && !st->error);
+      cudaGraphSetConditional(ctl.loop, !stop && !st->error);
+    }
   }
 }
 
 cudaError_t dense_qr_step(const double2* G, double2* C, double2* C_prev, double2* Sinv,
                           double2* SH, const double* bnorm, QrStepParams p, int N,
-                          SolverStatus* st, Gate gate, cudaStream_t s) {
+                          SolverStatus* st, Gate gate, LoopCtl ctl, cudaStream_t s) {
   size_t sm = 3ull * N * N * sizeof(double2);
   cudaFuncSetAttribute(k_dense_qr_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_dense_qr_step<<<1, DENSE_THREADS, sm, s>>>(G, C, C_prev, Sinv, SH, bnorm, p, N, st, gate);
+  k_dense_qr_step<<<1, DENSE_THREADS, sm, s>>>(G, C, C_prev, Sinv, SH, bnorm, p, N, st, gate, ctl);
   return cudaGetLastError();
 }
 
@@ -244,7 +262,7 @@ __global__ void __launch_bounds__(DENSE_THREADS)
                     double2* __restrict__ C_prev, double2* __restrict__ Cinv,
                     double2* __restrict__ SH, const double* __restrict__ bnorm,
                     double* __restrict__ tres_out, double tol, int init, int confirmed, int N,
-                    SolverStatus* st, Gate gate) {
+                    SolverStatus* st, Gate gate, LoopCtl ctl) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int flag;
   __shared__ double tres[64];
@@ -260,7 +278,10 @@ __global__ void __launch_bounds__(DENSE_THREADS)
   __syncthreads();
   int f = chol_lower(A, N, &flag);
   if (f) {
-    if (threadIdx.x == 0) st->error = f;
+    if (threadIdx.x == 0) {
+      st->error = f;
+      if (ctl.on) cudaGraphSetConditional(ctl.loop, 0);
+    }
     return;
   }
   tri_inv_lower(A, Wk, N);
@@ -301,6 +322,7 @@ __global__ void __launch_bounds__(DENSE_THREADS)
       if (confirmed) st->verified = 1;
     }
     if (!init) st->reliable_updates += 1;
+    if (ctl.on && (st->done || st->error)) cudaGraphSetConditional(ctl.loop, 0);
   }
 }
 
@@ -344,11 +366,12 @@ cudaError_t dense_verify(const double2* G, const double* bnorm, double* tres, do
 
 cudaError_t dense_restart(const double2* G, double2* C, double2* C_prev, double2* Cinv,
                           double2* SH, const double* bnorm, double* tres, double tol, int init,
-                          int confirmed, int N, SolverStatus* st, Gate gate, cudaStream_t s) {
+                          int confirmed, int N, SolverStatus* st, Gate gate, LoopCtl ctl,
+                          cudaStream_t s) {
   size_t sm = 3ull * N * N * sizeof(double2);
   cudaFuncSetAttribute(k_dense_restart, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   k_dense_restart<<<1, DENSE_THREADS, sm, s>>>(G, C, C_prev, Cinv, SH, bnorm, tres, tol, init,
-                                               confirmed, N, st, gate);
+                                               confirmed, N, st, gate, ctl);
   return cudaGetLastError();
 }
 
@@ -492,27 +515,6 @@ cudaError_t cg_restart_check(const double2* rr_sum, double* rr, double* beta, do
                              const double* bnorm, double n_elems, double tol, int init,
                              SolverStatus* st, cudaStream_t s) {
   k_cg_restart_check<<<1, 1, 0, s>>>(rr_sum, rr, beta, gam, bnorm, n_elems, tol, init, st);
-  return cudaGetLastError();
-}
-
-// Loop condition of a batched solve's device-side iteration loop (a CUDA
-// graph WHILE node): continue while the problem has neither converged,
-// failed nor used its iteration budget, and never beyond max_trips trips.
-__global__ void k_loop_condition(cudaGraphConditionalHandle handle, SolverStatus* st,
-                                 int max_trips) {
-  const int trips = st->trips + 1;
-  st->trips = trips;
-  unsigned go = (st->done || st->error || st->stopped) ? 0u : 1u;
-  if (trips >= max_trips) {
-    if (go) st->stopped = 1;
-    go = 0u;
-  }
-  cudaGraphSetConditional(handle, go);
-}
-
-cudaError_t loop_condition(cudaGraphConditionalHandle handle, SolverStatus* st, int max_trips,
-                           cudaStream_t s) {
-  k_loop_condition<<<1, 1, 0, s>>>(handle, st, max_trips);
   return cudaGetLastError();
 }
 

@@ -35,14 +35,22 @@ struct Gate {
   const SolverStatus* st;
   int mode;
   double thr;  // res_max threshold of GATE_RU_CHEAP / GATE_RU_FINE
+  bool rare;   // enqueued every iteration, but mostly closed
 };
 
-// launches gated on a pending reliable update are off in most iterations;
-// their launchers use persistent grids (a few blocks per SM) so that a
-// gated-off launch retires quickly
-inline bool gate_mostly_off(const Gate& g) {
-  return g.st && (g.mode == GATE_RU || g.mode == GATE_RU_CHEAP || g.mode == GATE_RU_FINE);
-}
+// host-enqueued launches gated on a pending reliable update are off in most
+// iterations; their launchers use persistent grids (a few blocks per SM) so
+// that a gated-off launch retires quickly
+inline bool gate_mostly_off(const Gate& g) { return g.rare; }
+
+// The device-looped iteration (build_loop in api.cu): the kernel that ends an
+// iteration sets the condition of the IF node around its reliable update
+// (`update`), and, with the update's last N x N kernel, that of the WHILE node
+// around the whole loop (`loop`).  on = 0: launched by the host, no nodes.
+struct LoopCtl {
+  cudaGraphConditionalHandle loop, update;
+  int on;
+};
 
 __device__ __forceinline__ bool gate_closed(const Gate& g) {
   if (g.mode == GATE_ALWAYS || g.st == nullptr) return false;
@@ -218,7 +226,7 @@ struct QrStepParams {
 };
 cudaError_t dense_qr_step(const double2* G, double2* C, double2* C_prev, double2* Sinv,
                           double2* SH, const double* bnorm, QrStepParams p, int N,
-                          SolverStatus* st, Gate gate, cudaStream_t s);
+                          SolverStatus* st, Gate gate, LoopCtl ctl, cudaStream_t s);
 // Cholesky of the true-residual Gram -> C_new, Cinv; convergence on the true
 // residual; S = C_new C_prev^-1 -> SH = S^dag (unless init).
 // tres (N doubles) receives the per-column true relative residuals;
@@ -226,7 +234,8 @@ cudaError_t dense_qr_step(const double2* G, double2* C, double2* C_prev, double2
 // shows is final (verified), else it awaits dense_verify.
 cudaError_t dense_restart(const double2* G, double2* C, double2* C_prev, double2* Cinv,
                           double2* SH, const double* bnorm, double* tres, double tol, int init,
-                          int confirmed, int N, SolverStatus* st, Gate gate, cudaStream_t s);
+                          int confirmed, int N, SolverStatus* st, Gate gate, LoopCtl ctl,
+                          cudaStream_t s);
 // native-FP64 confirmation of a convergence: true residuals from the FP64
 // Gram G of R = B - A Y into tres; verified, or done cleared and fp64_only set
 cudaError_t dense_verify(const double2* G, const double* bnorm, double* tres, double tol, int N,
@@ -253,11 +262,6 @@ cudaError_t cg_scalar_beta(const double2* rr_new_sum, double* rr, double* beta,
 cudaError_t cg_restart_check(const double2* rr_sum, double* rr, double* beta, double* gam,
                              const double* bnorm, double n_elems, double tol, int init,
                              SolverStatus* st, cudaStream_t s);
-
-// one-thread kernel ending a batched solve's device-side loop trip: sets the
-// WHILE condition to "not done, no error, not stopped" (stops after max_trips)
-cudaError_t loop_condition(cudaGraphConditionalHandle handle, SolverStatus* st, int max_trips,
-                           cudaStream_t s);
 
 // ---- grad.cu
 // gradient of a real loss with respect to the links (user layout [4][V][3][3],
