@@ -156,6 +156,83 @@ int gram_blocks(int N, int rows) {
   return b;
 }
 
+// The last step of the register-blocked Grams: the sum of each block entry
+// over the CTA's G row groups, written to the CTA's partial in a fixed order.
+// FP64 adds have a latency of 64 clocks here, so on small N, where G is large
+// (85 at N = 4, 256 at N = 1), one thread adding all groups in turn took 2 us an
+// entry; there (B <= 2) P neighbouring threads share a sum.  With B = 4 (N > 16,
+// G <= 17) one thread per block takes it, an entry at a time.
+// red: group_words(B) double2.
+constexpr int group_words(int B) { return (B <= 2 ? B : 1) * GRAM_THREADS; }
+
+template <class C, int B>
+__device__ __forceinline__ void reduce_groups(const cpx<typename C::acc> (&a)[B][B], bool active,
+                                              int NB, int G, int N, bool herm, int i0, int j0,
+                                              double2* red, double2* out) {
+  const int tid = threadIdx.x;
+  auto value = [&](int u, int v) {
+    return active ? make_double2(C::to_double(a[u][v].re), C::to_double(a[u][v].im))
+                  : make_double2(0.0, 0.0);
+  };
+  if constexpr (B > 2) {
+#pragma unroll
+    for (int u = 0; u < B; ++u)
+#pragma unroll
+      for (int v = 0; v < B; ++v) {
+        red[tid] = value(u, v);
+        __syncthreads();
+        if (tid < NB) {
+          double2 s = red[tid];
+          for (int g = 1; g < G; ++g) {
+            const double2 w = red[g * NB + tid];
+            s.x += w.x;
+            s.y += w.y;
+          }
+          if (i0 + u < N && j0 + v < N) out[(i0 + u) * N + (j0 + v)] = s;
+        }
+        __syncthreads();
+      }
+  } else {
+    const int nb = (N + B - 1) / B;
+    int P = 32;  // NB * B <= 128 for N <= 16
+    while (P > 1 && (NB * B * P > GRAM_THREADS || P > G)) P >>= 1;
+    const int e = tid / P, p = tid - e * P;
+    const int v = e / NB, b = e - v * NB;
+    int bi = 0, bj = b;
+    if (herm) {
+      int off = 0;
+      while (bi < nb && off + (nb - bi) <= b) {
+        off += nb - bi;
+        ++bi;
+      }
+      bj = bi + (b - off);
+    } else {
+      bi = b / nb;
+      bj = b - bi * nb;
+    }
+#pragma unroll
+    for (int u = 0; u < B; ++u) {
+#pragma unroll
+      for (int w = 0; w < B; ++w) red[w * GRAM_THREADS + tid] = value(u, w);
+      __syncthreads();
+      double sx = 0.0, sy = 0.0;
+      if (v < B)
+        for (int g = p; g < G; g += P) {
+          const double2 w = red[v * GRAM_THREADS + g * NB + b];
+          sx += w.x;
+          sy += w.y;
+        }
+      for (int o = P >> 1; o > 0; o >>= 1) {
+        sx += __shfl_xor_sync(0xffffffffu, sx, o);
+        sy += __shfl_xor_sync(0xffffffffu, sy, o);
+      }
+      const int i = bi * B + u, j = bj * B + v;
+      if (p == 0 && v < B && i < N && j < N) out[i * N + j] = make_double2(sx, sy);
+      __syncthreads();
+    }
+  }
+}
+
 // Register-blocked Gram: a CTA stages TS sites of X and Y in shared memory
 // (coalesced 128-bit loads of whole sites), then each thread accumulates a
 // B x B block of entries (i, j) over the rows of its row group, so every
@@ -231,53 +308,46 @@ __global__ void __launch_bounds__(GRAM_THREADS)
       }
     }
   }
-  // reduce the row groups of each block through shared memory, one entry of
-  // the B x B block at a time, and write this CTA's partial
   __syncthreads();
-  double2* red = reinterpret_cast<double2*>(smem_raw);
-  double2* out = partials + (long long)blockIdx.x * N * N;
-#pragma unroll
-  for (int u = 0; u < B; ++u)
-#pragma unroll
-    for (int v = 0; v < B; ++v) {
-      red[tid] = active ? make_double2(C::to_double(a[u][v].re), C::to_double(a[u][v].im))
-                        : make_double2(0.0, 0.0);
-      __syncthreads();
-      if (tid < NB) {
-        double2 sacc = red[tid];
-        for (int g2 = 1; g2 < G; ++g2) {
-          double2 w = red[g2 * NB + tid];
-          sacc.x += w.x;
-          sacc.y += w.y;
-        }
-        if (i0 + u < N && j0 + v < N) out[(i0 + u) * N + (j0 + v)] = sacc;
-      }
-      __syncthreads();
-    }
+  reduce_groups<C, B>(a, active, NB, G, N, herm, i0, j0, reinterpret_cast<double2*>(smem_raw),
+                      partials + (long long)blockIdx.x * N * N);
 }
 
-// warp per entry of the result (upper triangle when Hermitian); fixed
-// summation order over the per-CTA partials -> deterministic
-__global__ void k_gram_reduce(const double2* __restrict__ partials, int nblocks, int N, int herm,
-                              double2* __restrict__ out, Gate gate) {
+// one CTA per entry of the result (upper triangle when Hermitian); fixed
+// summation order over the per-CTA partials -> deterministic.  Bound by load
+// latency and the FP64 adds: a CTA per entry has all its loads in flight at
+// once and spreads the adds over the SMs (N = 16, 608 partials: 2.6 us; with a
+// warp per entry, 19 loads one after another, 10.8).
+static constexpr int REDUCE_THREADS = 128;
+
+__global__ void __launch_bounds__(REDUCE_THREADS)
+    k_gram_reduce(const double2* __restrict__ partials, int nblocks, int N, int herm,
+                  double2* __restrict__ out, Gate gate) {
+  __shared__ double2 sm[REDUCE_THREADS];
   if (gate_closed(gate)) return;
-  const int E = gram_entries(N, herm);
-  int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
-  if (warp >= E) return;
   int i, j;
-  entry_ij(warp, N, herm, i, j);
+  entry_ij(blockIdx.x, N, herm, i, j);
+  const double2* p = partials + i * N + j;
+  const long long st = (long long)N * N;
   double sx = 0.0, sy = 0.0;
-  for (int b = lane; b < nblocks; b += 32) {
-    double2 v = partials[(long long)b * N * N + i * N + j];
+#pragma unroll 4
+  for (int b = threadIdx.x; b < nblocks; b += REDUCE_THREADS) {
+    const double2 v = p[b * st];
     sx += v.x;
     sy += v.y;
+  }
+  sm[threadIdx.x] = make_double2(sx, sy);
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  for (int k = threadIdx.x + 32; k < REDUCE_THREADS; k += 32) {
+    sx += sm[k].x;
+    sy += sm[k].y;
   }
   for (int o = 16; o > 0; o >>= 1) {
     sx += __shfl_down_sync(0xffffffffu, sx, o);
     sy += __shfl_down_sync(0xffffffffu, sy, o);
   }
-  if (lane == 0) {
+  if (threadIdx.x == 0) {
     out[i * N + j] = make_double2(sx, (herm && i == j) ? 0.0 : sy);
     if (herm && i != j) out[j * N + i] = make_double2(sx, -sy);
   }
@@ -299,7 +369,7 @@ static void launch_gram_b(const void* X, const void* Y, int N, int Vh, int herm,
   int same = (X == Y);
   const int TS = gram_tile(tile, N, (same ? 1 : 2) * (size_t)N * 3 * sizeof(cpx<real>));
   size_t tiles = (same ? 1 : 2) * (size_t)TS * N * 3 * sizeof(cpx<real>);
-  size_t red = GRAM_THREADS * sizeof(double2);
+  size_t red = group_words(B) * sizeof(double2);
   size_t sm = tiles > red ? tiles : red;
   cudaFuncSetAttribute(k_gram<S, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   k_gram<S, B><<<nblocks, GRAM_THREADS, sm, s>>>((const typename S::elem*)X,
@@ -335,9 +405,8 @@ cudaError_t gram_partials(FieldKind k, const void* X, const void* Y, int N, int 
 
 cudaError_t gram_reduce(const double2* partials, int nblocks, int N, int hermitian, double2* out,
                         Gate gate, cudaStream_t s) {
-  int E = gram_entries(N, hermitian);
-  k_gram_reduce<<<nblk((long long)E * 32, 256), 256, 0, s>>>(partials, nblocks, N, hermitian, out,
-                                                             gate);
+  k_gram_reduce<<<gram_entries(N, hermitian), REDUCE_THREADS, 0, s>>>(partials, nblocks, N,
+                                                                      hermitian, out, gate);
   return cudaGetLastError();
 }
 
@@ -474,26 +543,8 @@ __global__ void __launch_bounds__(GRAM_THREADS)
     }
   }
   __syncthreads();
-  double2* red = reinterpret_cast<double2*>(smem_raw);
-  double2* out = partials + (long long)blockIdx.x * N * N;
-#pragma unroll
-  for (int u = 0; u < B; ++u)
-#pragma unroll
-    for (int v = 0; v < B; ++v) {
-      red[tid] = active ? make_double2(C::to_double(a[u][v].re), C::to_double(a[u][v].im))
-                        : make_double2(0.0, 0.0);
-      __syncthreads();
-      if (tid < NB) {
-        double2 sacc = red[tid];
-        for (int g2 = 1; g2 < G; ++g2) {
-          double2 w = red[g2 * NB + tid];
-          sacc.x += w.x;
-          sacc.y += w.y;
-        }
-        if (i0 + u < N && j0 + v < N) out[(i0 + u) * N + (j0 + v)] = sacc;
-      }
-      __syncthreads();
-    }
+  reduce_groups<C, B>(a, active, NB, G, N, true, i0, j0, reinterpret_cast<double2*>(smem_raw),
+                      partials + (long long)blockIdx.x * N * N);
 }
 
 template <class S, int B>
@@ -502,7 +553,7 @@ static void launch_w_gram_b(void* Q, const void* AP, const double2* beta, int N,
   using real = typename S::comp::real;
   const int TS = gram_tile(tile, N, 2 * (size_t)N * 3 * sizeof(cpx<real>));
   const size_t tiles = (2 * (size_t)TS * N * 3 + (size_t)N * N) * sizeof(cpx<real>);
-  const size_t red = GRAM_THREADS * sizeof(double2);
+  const size_t red = group_words(B) * sizeof(double2);
   const size_t sm = tiles > red ? tiles : red;
   cudaFuncSetAttribute(k_w_gram<S, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   k_w_gram<S, B><<<nblocks, GRAM_THREADS, sm, s>>>((typename S::elem*)Q,
