@@ -432,6 +432,8 @@ struct SolverStatus {
   int verified;        // 1: done rests on a native-FP64 true residual
   int fp64_only;       // 1: a double-float convergence failed its FP64
                        // confirmation; all later reliable updates are FP64
+  int arrivals;        // CTAs of the QR step that have finished (0 between calls)
+  double col_res[64];  // their columns' iterated relative residuals
 };
 
 }  // namespace bcg

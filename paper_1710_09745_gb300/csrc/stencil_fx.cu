@@ -39,26 +39,36 @@ __global__ void __launch_bounds__(256)
   const bool ok = e0 >= -90 && e0 <= 90;  // else the whole field goes to fx_plain
   const int e = ok ? e0 : 0;
   if (!ok && lane == 0) atomicOr(bad, 1u);
-  for (int i = lane; i < 144; i += 32) {
-    const int d = i / 9, c = (i % 9) / 3, j = i % 3;
-    const int en = 2 * (3 * (d >> 3) + j) + ((d >> 2) & 1), li = (d & 3) * 3 + c;
-    uint32_t w[4];
-    const double2 v = ok ? Ls[i] : make_double2(0.0, 0.0);
-    digit_words<4>(fixed_f64(v.x, e), fixed_f64(v.y, e), w);
+  // ten lanes per row colour c, so that a lane's column sums stay in registers
+  const int c = lane / 10;
+  int sum[8][2] = {};
+  if (c < 3)
+    for (int i = lane - 10 * c; i < 48; i += 10) {
+      const int d = i / 3, j = i - 3 * (i / 3);
+      const int en = 2 * (3 * (d >> 3) + j) + ((d >> 2) & 1), li = (d & 3) * 3 + c;
+      uint32_t w[4];
+      const double2 v = ok ? Ls[d * 9 + c * 3 + j] : make_double2(0.0, 0.0);
+      digit_words<4>(fixed_f64(v.x, e), fixed_f64(v.y, e), w);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const int wi = 3 * en + k;
-      rec[warp][((wi >> 1) * 12 + li) * 2 + (wi & 1)] = w[k];
+      for (int k = 0; k < 3; ++k) {
+        const int wi = 3 * en + k;
+        rec[warp][((wi >> 1) * 12 + li) * 2 + (wi & 1)] = w[k];
+      }
+      rec[warp][REC_DIG / 4 + ((en >> 1) * 12 + li) * 2 + (en & 1)] = w[3];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        const uint32_t b = w[t >> 1] >> (16 * (t & 1));
+        const int re = (int)(b & 255u) - 128, im = (int)((b >> 8) & 255u) - 128;
+        sum[t][0] += re - im;  // column (c, re): Re, -Im
+        sum[t][1] += re + im;  // column (c, im): Im, Re
+      }
     }
-    rec[warp][REC_DIG / 4 + ((en >> 1) * 12 + li) * 2 + (en & 1)] = w[3];
+  if (c < 3)
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-      const uint32_t b = w[t >> 1] >> (16 * (t & 1));
-      const int re = (int)(b & 255u) - 128, im = (int)((b >> 8) & 255u) - 128;
-      atomicAdd(&sums[warp][c][t][0], re - im);  // column (c, re): Re, -Im
-      atomicAdd(&sums[warp][c][t][1], re + im);  // column (c, im): Im, Re
+      atomicAdd(&sums[warp][c][t][0], sum[t][0]);
+      atomicAdd(&sums[warp][c][t][1], sum[t][1]);
     }
-  }
   __syncwarp();
   const long long ps = (long long)p * g.Vh + site;
   uint32_t* om = reinterpret_cast<uint32_t*>(main + ps * REC_MAIN);
@@ -67,16 +77,16 @@ __global__ void __launch_bounds__(256)
   for (int i = lane; i < REC_EXTRA / 4; i += 32) ox[i] = rec[warp][REC_DIG / 4 + i];
   float* oi = reinterpret_cast<float*>(main + ps * REC_MAIN + REC_DIG);
   for (int i = lane; i < 48; i += 32) {
-    const int c = i / 16, u = (i / 2) & 7, part = i & 1;
-    int sum = 0;
-    for (int t = 0; t <= u; ++t) sum += sums[warp][c][t][part];
-    oi[i] = -1.490116119384765625e-08f * (float)sum;  // 128 * 2^-24 * 2^-9 = 2^-26
+    const int cc = i / 16, u = (i / 2) & 7, part = i & 1;
+    int tot = 0;
+    for (int t = 0; t <= u; ++t) tot += sums[warp][cc][t][part];
+    oi[i] = -1.490116119384765625e-08f * (float)tot;  // 128 * 2^-24 * 2^-9 = 2^-26
   }
   if (lane < 6) {  // double-float's D_6: the kept products only
-    int sum = 0;
+    int tot = 0;
     for (int t = 0; t < 6; ++t)
-      if (keep<6>(6 - t, t)) sum += sums[warp][lane / 2][t][lane & 1];
-    oi[48 + lane] = -1.490116119384765625e-08f * (float)sum;
+      if (keep<6>(6 - t, t)) tot += sums[warp][lane / 2][t][lane & 1];
+    oi[48 + lane] = -1.490116119384765625e-08f * (float)tot;
   }
   if (lane == 0) reinterpret_cast<int*>(oi)[54] = e;
 }
