@@ -405,11 +405,17 @@ int stencil_R(blockcg_ctx* h, FieldKind k, int N, const void* links, const void*
     return best;
   }
   Gate g0{nullptr, GATE_ALWAYS};
-  const int cands[13] = {1, 2, 4, 8, 1 | DSLASH_TMA, 2 | DSLASH_TMA, 4 | DSLASH_TMA, 8 | DSLASH_TMA,
+  const int cands[15] = {1, 2, 4, 8, 1 | DSLASH_TMA, 2 | DSLASH_TMA, 4 | DSLASH_TMA, 8 | DSLASH_TMA,
                          1 | DSLASH_ASYNC, 2 | DSLASH_ASYNC, 4 | DSLASH_ASYNC, 8 | DSLASH_ASYNC,
-                         1 | DSLASH_TC};
+                         1 | DSLASH_TC, 4 | DSLASH_SPLIT, 16 | DSLASH_SPLIT};
   for (int R : cands) {
-    if ((R & 0xff) > 1 && (R & 0xff) > N) continue;
+    if ((R & 0xff) > 1 && (R & 0xff) > N && !(R & DSLASH_SPLIT)) continue;
+    // hop-split: full links, and few enough outputs that splitting can pay
+    // (at 16^4, N = 1 a half takes 22 us against 26, at 4^4, N = 4 it is 4
+    // against 14; from 2^15 outputs on the other kernels fill the GPU)
+    if ((R & DSLASH_SPLIT) &&
+        (rf || k == FK_H16 || k == FK_BF16 || (long long)h->g.Vh * N > 1 << 15))
+      continue;
     // the tensor-core stencil: double-float and FP64, and FP16 and bfloat16
     // with N = 16 or 32 and full links
     if ((R & DSLASH_TC) &&
@@ -417,7 +423,7 @@ int stencil_R(blockcg_ctx* h, FieldKind k, int N, const void* links, const void*
                  ((k == FK_H16 || k == FK_BF16) && dslash_tc16_supported(N)))))
       continue;
     if (rf) {  // two-row links: the plain kernel only
-      if (R & (DSLASH_TMA | DSLASH_ASYNC)) continue;
+      if (R & (DSLASH_TMA | DSLASH_ASYNC | DSLASH_SPLIT)) continue;
       R |= rf;
     }
     // double-float with N >= 2: the cp.async kernel only.  Timed alone the
@@ -425,7 +431,7 @@ int stencil_R(blockcg_ctx* h, FieldKind k, int N, const void* links, const void*
     // Gram, N x N and update kernels) it ran 12-15 % slower than that timing
     // in repeated 32^4 N = 16 measurements, while the cp.async kernel ran as
     // timed.
-    if (k == FK_DF && N >= 2 && !(R & (DSLASH_ASYNC | DSLASH_TC))) continue;
+    if (k == FK_DF && N >= 2 && !(R & (DSLASH_ASYNC | DSLASH_TC | DSLASH_SPLIT))) continue;
     if (fx_only(h, k, N) && !(R & DSLASH_TC)) continue;
     const double m2 = h->mass * h->mass;
     auto run = [&]() {
@@ -436,15 +442,22 @@ int stencil_R(blockcg_ctx* h, FieldKind k, int N, const void* links, const void*
                    g0, h->stream);
       return e;
     };
+    // one run first (after the first candidate a run that takes more than
+    // twice the best settles it), then three
+    float ms = 0.f;
+    cudaEventRecord(e0, h->stream);
     if (run() != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
+    cudaEventRecord(e1, h->stream);
+    if (cudaEventSynchronize(e1) != cudaSuccess) continue;
+    cudaEventElapsedTime(&ms, e0, e1);
+    if (ms * 3.f > 2.f * best_ms && ms > 0.02f) continue;
     cudaEventRecord(e0, h->stream);
     for (int i = 0; i < 3; ++i) run();
     cudaEventRecord(e1, h->stream);
     if (cudaEventSynchronize(e1) != cudaSuccess) continue;
-    float ms = 0.f;
     cudaEventElapsedTime(&ms, e0, e1);
     if (ms < best_ms) {
       best_ms = ms;

@@ -104,6 +104,9 @@ static constexpr int DSLASH_TC = 0x2000;
 // the other kernels ignore both flags)
 static constexpr int DSLASH_FIRST = 0x4000;
 static constexpr int DSLASH_SECOND = 0x8000;
+// R | DSLASH_SPLIT, R = 4 or 16 lanes per output: the hop-split kernel
+// (full links, 32- and 64-bit kinds; an autotuner candidate on small problems)
+static constexpr int DSLASH_SPLIT = 0x10000;
 bool dslash_fx_supported(const Geom& g, int N);
 size_t fx_links_bytes(const Geom& g);
 size_t fx_digit_bytes(const Geom& g, int N);

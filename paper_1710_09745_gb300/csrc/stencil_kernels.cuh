@@ -877,6 +877,119 @@ static void launch_dslash_s(int R, int epi, const void* links, const void* in, v
 }
 
 
+// ---------------------------------------------------------------------------
+// Hop-split stencil for problems too small to fill the GPU: HS lanes share an
+// output (site, right-hand side), each taking 16 / HS hops (HS = 4: the hops of
+// one direction, HS = 16: one hop), and add their partial sums by shuffles;
+// lane h < 3 of the group finishes and writes colour h.  Such a problem is
+// bound by the chain of one thread (a double-float hop is 432 dependent-ish
+// FP32 instructions behind its loads), which this shortens HS-fold for
+// log2(HS) steps of shuffles; the autotuner takes it where that is faster.
+// A warp's lanes: 32 / HS neighbouring outputs for each part, so that the loads
+// of one part run over consecutive right-hand sides.
+template <class C>
+__device__ __forceinline__ void acc_join(typename C::acc& a, int o) {
+  if constexpr (std::is_same<C, CompDF>::value) {
+    const dfacc b{__shfl_xor_sync(0xffffffffu, a.s, o), __shfl_xor_sync(0xffffffffu, a.e, o)};
+    float s, e;
+    two_sum(a.s, b.s, s, e);
+    a = {s, __fadd_rn(__fadd_rn(a.e, b.e), e)};
+  } else {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+  }
+}
+
+template <class S, int HS, int EPI>
+__global__ void __launch_bounds__(128)
+    k_dslash_split(const typename S::elem* __restrict__ links, const typename S::elem* __restrict__ in,
+                   typename S::elem* __restrict__ out, const typename S::elem* __restrict__ c1,
+                   const typename S::elem* __restrict__ c2, double m2d, Geom g, int parity, int N,
+                   Gate gate) {
+  using C = typename S::comp;
+  using real = typename C::real;
+  using acc = typename C::acc;
+  if (gate_closed(gate)) return;
+  constexpr int PER = 32 / HS;  // outputs per warp
+  const int lane = threadIdx.x & 31, h = lane / PER;
+  const real m2 = C::from_double(m2d);
+  const long long total = (long long)g.Vh * N;
+  const long long warps = (total + PER - 1) / PER;
+  for (long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < warps;
+       w += (long long)gridDim.x * (blockDim.x >> 5)) {
+    const long long gid = min(w * PER + lane % PER, total - 1);  // past the end: repeat the last
+    const int site = (int)(gid / N);
+    const int n = (int)(gid - (long long)site * N);
+    int x, y, z, t;
+    site_xyzt(g, site, parity, x, y, z, t);
+    const int lex = x + g.L[0] * (y + g.L[1] * (z + g.L[2] * t));
+    cpx<acc> a[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) a[i] = czero<C>();
+    const typename S::elem* lp = links + link_offset(g, parity, site);
+#pragma unroll
+    for (int q = 0; q < 16 / HS; ++q) {
+      const int d = h * (16 / HS) + q;
+      const int nb = neighbour_cb_s(g, lex, x, y, z, t, d >> 2, hop_k(d & 3));
+      const typename S::elem* ip = in + (long long)nb * N * 3 + n;
+      cpx<real> v[3], U[9];
+#pragma unroll
+      for (int b = 0; b < 3; ++b) v[b] = S::load_raw(ip + b * N);
+#pragma unroll
+      for (int e = 0; e < 9; ++e) U[e] = S::load_raw(lp + (d * 9 + e) * LINK_W);
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) cmac<C>(a[i], U[i * 3 + b], v[b]);
+    }
+#pragma unroll
+    for (int o = PER; o < 32; o <<= 1)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        acc_join<C>(a[i].re, o);
+        acc_join<C>(a[i].im, o);
+      }
+    if (h < 3 && w * PER + lane % PER < total) {
+      cpx<acc> v = h == 0 ? a[0] : h == 1 ? a[1] : a[2];
+      unscale_raw<S>(v);
+      const long long oi = ((long long)site * 3 + h) * N + n;
+      if (EPI != EPI_NONE) {
+        C::neg(v.re);
+        C::neg(v.im);
+        const cpx<real> cc = S::load(c1 + oi);
+        C::mac(v.re, m2, cc.re);
+        C::mac(v.im, m2, cc.im);
+        if (EPI == EPI_RESIDUAL) {
+          C::neg(v.re);
+          C::neg(v.im);
+          const cpx<real> bb = S::load(c2 + oi);
+          C::add(v.re, bb.re);
+          C::add(v.im, bb.im);
+        }
+      }
+      S::store(out + oi, cfin<C>(v));
+    }
+  }
+}
+
+template <class S, int HS>
+static void launch_split(int epi, const void* links, const void* in, void* out, const void* c1,
+                         const void* c2, double m2, const Geom& g, int parity, int N, Gate gate,
+                         cudaStream_t s) {
+  using E = typename S::elem;
+  const long long warps = ((long long)g.Vh * N + 32 / HS - 1) / (32 / HS);
+  const long long want = (warps + 3) / 4, cap = (long long)stencil_sms() * (gate_mostly_off(gate) ? 4 : 64);
+  const unsigned blocks = (unsigned)(want < cap ? want : cap);
+  auto run = [&](auto kern) {
+    kern<<<blocks, 128, 0, s>>>((const E*)links, (const E*)in, (E*)out, (const E*)c1, (const E*)c2,
+                                m2, g, parity, N, gate);
+  };
+  switch (epi) {
+    case EPI_NONE: run(k_dslash_split<S, HS, EPI_NONE>); break;
+    case EPI_NORMAL: run(k_dslash_split<S, HS, EPI_NORMAL>); break;
+    default: run(k_dslash_split<S, HS, EPI_RESIDUAL>); break;
+  }
+}
+
 // One storage kind: the cp.async prefetch kernel (R | DSLASH_ASYNC), the
 // bulk-copy pipelined kernel (R | DSLASH_TMA) or the plain kernel; a
 // pipelined request that cannot run for this N falls back to the plain one.
@@ -891,6 +1004,15 @@ static cudaError_t dslash_kind(int R, int epi, const void* links, const void* in
       return cudaGetLastError();
     } else {
       return cudaErrorInvalidValue;
+    }
+  }
+  if constexpr (!std::is_same<S, StoreH16>::value && !std::is_same<S, StoreBF16>::value) {
+    if (R & DSLASH_SPLIT) {
+      if ((R & 0xff) == 16)
+        launch_split<S, 16>(epi, links, in, out, c1, c2, m2, g, out_parity, N, gate, s);
+      else
+        launch_split<S, 4>(epi, links, in, out, c1, c2, m2, g, out_parity, N, gate, s);
+      return cudaGetLastError();
     }
   }
   if (R & DSLASH_ASYNC) {
