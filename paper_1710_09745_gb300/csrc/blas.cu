@@ -46,50 +46,71 @@ static inline unsigned gcap(long long n, int t, unsigned cap = 152 * 8) {
 }
 
 // ------------------------------------------------------------ layout ----
+// A tile of LT sites and up to LJ columns goes through shared memory, so that
+// both sides are read and written in runs: LT * 3 numbers of one column on the
+// user's side, the LJ columns of a row on the internal one.
+static constexpr int LT = 32, LJ = 16, LP = LT * 3 + 1;
+
 template <class S>
-__global__ void k_to_internal(const double2* __restrict__ user, typename S::elem* __restrict__ in,
-                              int N, int Vh) {
-  long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  long long total = (long long)Vh * N * 3;
-  if (idx >= total) return;
-  int j = (int)(idx % N);
-  long long t = idx / N;
-  int c = (int)(t % 3);
-  long long site = t / 3;
-  in[idx] = S::from_double2(user[((long long)j * Vh + site) * 3 + c]);
+__global__ void __launch_bounds__(256)
+    k_to_internal(const double2* __restrict__ user, typename S::elem* __restrict__ in, int N,
+                  int Vh) {
+  __shared__ typename S::elem tile[LJ * LP];
+  const long long s0 = (long long)blockIdx.x * LT;
+  const int j0 = blockIdx.y * LJ, nj = min(LJ, N - j0);
+  const int rows = (int)min((long long)LT, Vh - s0) * 3;
+  for (int idx = threadIdx.x; idx < nj * LT * 3; idx += 256) {
+    const int j = idx / (LT * 3), r = idx - j * (LT * 3);
+    if (r < rows) tile[j * LP + r] = S::from_double2(user[((j0 + j) * (long long)Vh + s0) * 3 + r]);
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < nj * rows; idx += 256) {
+    const int r = idx / nj, j = idx - r * nj;
+    in[(s0 * 3 + r) * N + j0 + j] = tile[j * LP + r];
+  }
 }
 
 template <class S>
-__global__ void k_from_internal(const typename S::elem* __restrict__ in, double2* __restrict__ user,
-                                int N, int Vh) {
-  long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  long long total = (long long)Vh * N * 3;
-  if (idx >= total) return;
-  int j = (int)(idx % N);
-  long long t = idx / N;
-  int c = (int)(t % 3);
-  long long site = t / 3;
-  user[((long long)j * Vh + site) * 3 + c] = S::to_double2(in[idx]);
+__global__ void __launch_bounds__(256)
+    k_from_internal(const typename S::elem* __restrict__ in, double2* __restrict__ user, int N,
+                    int Vh) {
+  __shared__ typename S::elem tile[LJ * LP];
+  const long long s0 = (long long)blockIdx.x * LT;
+  const int j0 = blockIdx.y * LJ, nj = min(LJ, N - j0);
+  const int rows = (int)min((long long)LT, Vh - s0) * 3;
+  for (int idx = threadIdx.x; idx < nj * rows; idx += 256) {
+    const int r = idx / nj, j = idx - r * nj;
+    tile[j * LP + r] = in[(s0 * 3 + r) * N + j0 + j];
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < nj * LT * 3; idx += 256) {
+    const int j = idx / (LT * 3), r = idx - j * (LT * 3);
+    if (r < rows) user[((j0 + j) * (long long)Vh + s0) * 3 + r] = S::to_double2(tile[j * LP + r]);
+  }
+}
+
+static dim3 layout_grid(int N, int Vh) {
+  return dim3((unsigned)((Vh + LT - 1) / LT), (unsigned)((N + LJ - 1) / LJ));
 }
 
 cudaError_t to_internal(FieldKind k, const double2* user, void* internal, int N, int Vh,
                         cudaStream_t s) {
-  long long total = (long long)Vh * N * 3;
+  const dim3 grid = layout_grid(N, Vh);
   switch (k) {
     case FK_DF:
-      k_to_internal<StoreDF><<<nblk(total, 256), 256, 0, s>>>(user, (float4*)internal, N, Vh);
+      k_to_internal<StoreDF><<<grid, 256, 0, s>>>(user, (float4*)internal, N, Vh);
       break;
     case FK_F32:
-      k_to_internal<StoreF32><<<nblk(total, 256), 256, 0, s>>>(user, (float2*)internal, N, Vh);
+      k_to_internal<StoreF32><<<grid, 256, 0, s>>>(user, (float2*)internal, N, Vh);
       break;
     case FK_F64:
-      k_to_internal<StoreF64><<<nblk(total, 256), 256, 0, s>>>(user, (double2*)internal, N, Vh);
+      k_to_internal<StoreF64><<<grid, 256, 0, s>>>(user, (double2*)internal, N, Vh);
       break;
     case FK_H16:
-      k_to_internal<StoreH16><<<nblk(total, 256), 256, 0, s>>>(user, (__half2*)internal, N, Vh);
+      k_to_internal<StoreH16><<<grid, 256, 0, s>>>(user, (__half2*)internal, N, Vh);
       break;
     case FK_BF16:
-      k_to_internal<StoreBF16><<<nblk(total, 256), 256, 0, s>>>(user, (__nv_bfloat162*)internal, N, Vh);
+      k_to_internal<StoreBF16><<<grid, 256, 0, s>>>(user, (__nv_bfloat162*)internal, N, Vh);
       break;
   }
   return cudaGetLastError();
@@ -97,22 +118,22 @@ cudaError_t to_internal(FieldKind k, const double2* user, void* internal, int N,
 
 cudaError_t from_internal(FieldKind k, const void* internal, double2* user, int N, int Vh,
                           cudaStream_t s) {
-  long long total = (long long)Vh * N * 3;
+  const dim3 grid = layout_grid(N, Vh);
   switch (k) {
     case FK_DF:
-      k_from_internal<StoreDF><<<nblk(total, 256), 256, 0, s>>>((const float4*)internal, user, N, Vh);
+      k_from_internal<StoreDF><<<grid, 256, 0, s>>>((const float4*)internal, user, N, Vh);
       break;
     case FK_F32:
-      k_from_internal<StoreF32><<<nblk(total, 256), 256, 0, s>>>((const float2*)internal, user, N, Vh);
+      k_from_internal<StoreF32><<<grid, 256, 0, s>>>((const float2*)internal, user, N, Vh);
       break;
     case FK_F64:
-      k_from_internal<StoreF64><<<nblk(total, 256), 256, 0, s>>>((const double2*)internal, user, N, Vh);
+      k_from_internal<StoreF64><<<grid, 256, 0, s>>>((const double2*)internal, user, N, Vh);
       break;
     case FK_H16:
-      k_from_internal<StoreH16><<<nblk(total, 256), 256, 0, s>>>((const __half2*)internal, user, N, Vh);
+      k_from_internal<StoreH16><<<grid, 256, 0, s>>>((const __half2*)internal, user, N, Vh);
       break;
     case FK_BF16:
-      k_from_internal<StoreBF16><<<nblk(total, 256), 256, 0, s>>>((const __nv_bfloat162*)internal, user, N, Vh);
+      k_from_internal<StoreBF16><<<grid, 256, 0, s>>>((const __nv_bfloat162*)internal, user, N, Vh);
       break;
   }
   return cudaGetLastError();

@@ -32,13 +32,45 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
 }
 
+// Conversions between double and double-float on the integer and FP32 pipes:
+// as FP64 adds and format conversions they bound the kernels that convert
+// whole fields (32^4, N = 16: 359 us for a layout conversion whose bytes take
+// 121).  hi is the value rounded to 24 bits, lo the remainder rounded to 24
+// bits, as x - (double)hi gives it; outside 2^-90 .. 2^90, and for zeros, infinities
+// and NaN, the FP64 operations themselves (out of line, or the compiler would
+// execute both sides).
+__device__ __noinline__ inline df df_from_double_fp64(double x) {
+  const float h = __double2float_rn(x);
+  return {h, __double2float_rn(x - (double)h)};
+}
 __device__ __forceinline__ df df_from_double(double x) {
-  float h = __double2float_rn(x);
-  float l = __double2float_rn(x - (double)h);
-  return {h, l};
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ff) - 1023;
+  if (e < -90 || e > 90) return df_from_double_fp64(x);
+  const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+  const unsigned h = (unsigned)((m + (1ull << 28)) >> 29);      // to 24 bits
+  const int r = (int)((unsigned)m - (h << 29));                 // |r| <= 2^28
+  const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+  const float u = __uint_as_float(sign | (unsigned)((e + 127 - 23) << 23));  // +-2^(e - 23)
+  const float hi = __fmul_rn(__uint2float_rn(h), u);
+  return {hi, __fmul_rn(__int2float_rn(r), __fmul_rn(u, 1.862645149230957e-09f))};  // 2^-29
 }
 
-__device__ __forceinline__ double df_to_double(df a) { return (double)a.hi + (double)a.lo; }
+__device__ __noinline__ inline double df_to_double_fp64(df a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double df_to_double(df a) {
+  const unsigned b = __float_as_uint(a.hi), c = __float_as_uint(a.lo);
+  const int e = (int)((b >> 23) & 0xff) - 127, le = (int)((c >> 23) & 0xff) - 127;
+  if (e < -90 || e > 90 || le > e - 24) return df_to_double_fp64(a);
+  // lo in units of 2^(e - 52), the result's last place (|lo| <= ulp(hi) / 2)
+  const int sh = e - 29 - le;  // >= -5
+  const unsigned ml = (c & 0x7fffffu) | 0x800000u;
+  const unsigned r = sh <= 0 ? ml << -sh : sh > 25 ? 0u : (ml + (1u << (sh - 1))) >> sh;
+  unsigned long long m = (unsigned long long)((b & 0x7fffffu) | 0x800000u) << 29;
+  m = ((b ^ c) >> 31) ? m - r : m + r;
+  if (m < 0x10000000000000ull) return df_to_double_fp64(a);  // hi a power of two, lo < 0
+  return __longlong_as_double((long long)(((unsigned long long)(b & 0x80000000u) << 32) +
+                                          ((unsigned long long)(e + 1022) << 52) + m));
+}
 
 // accumulator: value = s + e, e not normalised
 struct dfacc {
@@ -186,7 +218,7 @@ struct StoreDF {  // {re.hi, im.hi, re.lo, im.lo}: one 128-bit word per complex
     return make_float4(r.hi, i.hi, r.lo, i.lo);
   }
   static __device__ __forceinline__ double2 to_double2(elem v) {
-    return make_double2((double)v.x + (double)v.z, (double)v.y + (double)v.w);
+    return make_double2(df_to_double({v.x, v.z}), df_to_double({v.y, v.w}));
   }
 };
 

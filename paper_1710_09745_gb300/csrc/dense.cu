@@ -168,8 +168,7 @@ __device__ void load_mat(double2* dst, const double2* __restrict__ src, int N) {
 
 // s += a b
 __device__ __forceinline__ void cmad(double2& s, double2 a, double2 b) {
-  s.x = fma(a.x, b.x, fma(-a.y, b.y, s.x));
-  s.y = fma(a.x, b.y, fma(a.y, b.x, s.y));
+  s = cadd(s, cm(a, b));
 }
 // sum over the n (a power of two) neighbouring lanes that share a row
 __device__ __forceinline__ double2 lane_sum(double2 s, int n) {
