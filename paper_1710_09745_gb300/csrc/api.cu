@@ -581,7 +581,9 @@ void tune_blas(blockcg_ctx* h, const Ws& w, int N) {
                            WG_TC);
     });
     if (t < t_wgram) t_wgram = t, best_wgram = WG_TC;
-    t = time3([&] {
+  }
+  if (gram_tc_supported(k, N)) {
+    float t = time3([&] {
       return gram_partials(k, w.AP, w.Ts, N, Vh, 1, w.partials, w.nblocks, g0, s, GR_TC);
     });
     if (t < t_gram) t_gram = t, best_gram = GR_TC;

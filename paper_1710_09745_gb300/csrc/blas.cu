@@ -411,7 +411,7 @@ static void launch_gram(const void* X, const void* Y, int N, int Vh, int herm, d
 
 cudaError_t gram_partials(FieldKind k, const void* X, const void* Y, int N, int Vh, int hermitian,
                           double2* partials, int nblocks, Gate gate, cudaStream_t s, int tile) {
-  if ((tile & GR_TC) && hermitian && w_gram_tc_supported(k, N))
+  if ((tile & GR_TC) && hermitian && gram_tc_supported(k, N))
     return gram_partials_tc(k, X, Y, N, Vh, partials, nblocks, gate, s);
   tile &= ~GR_TC;
   switch (k) {
@@ -992,9 +992,9 @@ static cudaError_t launch_bcg_update(void* Q, void* P, void* X, const double2* S
 
 cudaError_t bcg_update(FieldKind sk, FieldKind xk, void* Q, void* P, void* X, const double2* Sinv,
                        const double2* BC, const double2* SH, int N, int Vh, Gate gate,
-                       cudaStream_t s, int tile) {
+                       cudaStream_t s, int tile, unsigned* pmax) {
   if ((tile & UPD_TC) && bcg_update_tc_supported(sk, xk, N))
-    return bcg_update_tc(sk, Q, P, X, Sinv, BC, SH, N, Vh, gate, s);
+    return bcg_update_tc(sk, Q, P, X, Sinv, BC, SH, N, Vh, pmax, gate, s);
   tile &= ~UPD_TC;
   if (sk == FK_DF && xk == FK_DF)
     return launch_bcg_update<StoreDF, StoreDF>(Q, P, X, Sinv, BC, SH, N, Vh, gate, tile, s);

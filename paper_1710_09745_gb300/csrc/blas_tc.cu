@@ -406,7 +406,7 @@ __device__ __forceinline__ void gram_tc_tile(const uint32_t* sX, const uint32_t*
 template <int N, bool HERM>
 __device__ __forceinline__ void gram_tc_write(double2* out,
                                               const dfacc (&gacc)[GramBlocks<N, HERM>::PER_WARP][4],
-                                              double scale, int warp, int lane) {
+                                              double scale, int warp, int lane, int n = N) {
   using GB = GramBlocks<N, HERM>;
   const int g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -425,10 +425,10 @@ __device__ __forceinline__ void gram_tc_write(double2* out,
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int i = 8 * mt + (g >> 1) + 4 * h;
-        if (!HERM || i <= j) {
+        if ((!HERM || i <= j) && i < n && j < n) {
           const double kre = v[2 * h] + p[2 * h + 1];
           const double kim = v[2 * h + 1] - p[2 * h];
-          out[i * N + j] = make_double2(kre * scale, kim * scale);
+          out[i * n + j] = make_double2(kre * scale, kim * scale);
         }
       }
     }
@@ -633,10 +633,11 @@ static cudaError_t launch_gram_tc(const void* X, const void* Y, int Vh, double2*
 }
 
 // ---------------------------------------------------------------------------
-// K = X^dag Y for the double-float kind (N = 16) on the tensor cores, as exact
+// K = X^dag Y for the double-float and the FP32 kind on the tensor cores, as exact
 // split products (ozaki.cuh): per CTA tile of TGD = 64 rows, every column of X
 // and of Y gets a power-of-two scale from its largest entry in the tile
-// (shared-memory maxima), each scaled value is split into six bf16 slices,
+// (shared-memory maxima), each scaled value is split into six bf16 slices (four
+// for FP32, with 9 to 32 columns, the tiles padded with zeros to NP = 16 or 32),
 // and slice s of a tile is stored like the 16-bit tiles above ([row][RW]
 // words of (re, im) pairs).  A warp's Gram block accumulates the products of
 // slices s, t with s + t = u in D_u: over the tile's 64 rows the terms share
@@ -647,13 +648,16 @@ static cudaError_t launch_gram_tc(const void* X, const void* Y, int Vh, double2*
 // i <= j; X == Y (a Gram of one block) stages one set of slices.
 constexpr int TGD = 64;  // rows per CTA tile
 
-template <int N, bool SAME>
-__global__ void __launch_bounds__(TC_WARPS * 32, N == 16 ? (SAME ? 3 : 2) : 1)
-    k_gram_tc_df(const float4* __restrict__ X, const float4* __restrict__ Y, int Vh,
-                 double2* __restrict__ partials, Gate gate) {
+template <class S, int NP, bool SAME>
+__global__ void __launch_bounds__(TC_WARPS * 32, NP == 16 ? (SAME ? 3 : 2) : 1)
+    k_gram_tc_df(const typename S::elem* __restrict__ X, const typename S::elem* __restrict__ Y,
+                 int n, int Vh, double2* __restrict__ partials, Gate gate) {
+  using K = ozaki::SliceKind<S>;
+  using E = typename S::elem;
+  constexpr int N = NP;  // columns of a tile, of which n are used
   using GB = GramBlocks<N, true>;
   constexpr int RW = N + 4;
-  constexpr int NSL = 6;
+  constexpr int NSL = K::NSL;
   constexpr int PER = TGD * N / (TC_WARPS * 32);  // entries of a tile per thread
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint32_t* sX = reinterpret_cast<uint32_t*>(smem_raw);  // [NSL][TGD][RW]
@@ -671,21 +675,21 @@ __global__ void __launch_bounds__(TC_WARPS * 32, N == 16 ? (SAME ? 3 : 2) : 1)
   for (long long tile = blockIdx.x; tile * TGD < nrows; tile += gridDim.x) {
     if (threadIdx.x < N) sMx[threadIdx.x] = sMy[threadIdx.x] = 0u;
     __syncthreads();  // also: the previous tile's slices have been read
-    float4 xv[PER], yv[PER];
+    E xv[PER], yv[PER];
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
       const int idx = threadIdx.x + k * TC_WARPS * 32;  // column idx % N (N divides 256)
       const long long r = tile * TGD + idx / N;
-      const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-      xv[k] = r < nrows ? X[r * N + idx % N] : z;
-      yv[k] = SAME ? xv[k] : (r < nrows ? Y[r * N + idx % N] : z);
+      const bool ok = r < nrows && idx % N < n;
+      xv[k] = ok ? X[r * n + idx % N] : K::zero();
+      yv[k] = SAME ? xv[k] : ok ? Y[r * n + idx % N] : K::zero();
     }
     {
       float mx = 0.f, my = 0.f;
 #pragma unroll
       for (int k = 0; k < PER; ++k) {
-        mx = fmaxf(mx, fmaxf(fabsf(xv[k].x), fabsf(xv[k].y)));
-        my = fmaxf(my, fmaxf(fabsf(yv[k].x), fabsf(yv[k].y)));
+        mx = fmaxf(mx, K::mag(xv[k]));
+        my = fmaxf(my, K::mag(yv[k]));
       }
       atomicMax(&sMx[threadIdx.x % N], __float_as_uint(mx));
       if (!SAME) atomicMax(&sMy[threadIdx.x % N], __float_as_uint(my));
@@ -702,18 +706,14 @@ __global__ void __launch_bounds__(TC_WARPS * 32, N == 16 ? (SAME ? 3 : 2) : 1)
 #pragma unroll
       for (int k = 0; k < PER; ++k) {
         const int row = (threadIdx.x + k * TC_WARPS * 32) / N;
-        float sr[NSL], si[NSL];
-        ozaki::split6(__fmul_rn(xv[k].x, scx), __fmul_rn(xv[k].z, scx), sr);
-        ozaki::split6(__fmul_rn(xv[k].y, scx), __fmul_rn(xv[k].w, scx), si);
+        uint32_t w[NSL];
+        K::slices(xv[k], scx, w);
 #pragma unroll
-        for (int sl = 0; sl < NSL; ++sl)
-          sX[(sl * TGD + row) * RW + c] = ozaki::pack_bf16(sr[sl], si[sl]);
+        for (int sl = 0; sl < NSL; ++sl) sX[(sl * TGD + row) * RW + c] = w[sl];
         if (!SAME) {
-          ozaki::split6(__fmul_rn(yv[k].x, scy), __fmul_rn(yv[k].z, scy), sr);
-          ozaki::split6(__fmul_rn(yv[k].y, scy), __fmul_rn(yv[k].w, scy), si);
+          K::slices(yv[k], scy, w);
 #pragma unroll
-          for (int sl = 0; sl < NSL; ++sl)
-            sY[(sl * TGD + row) * RW + c] = ozaki::pack_bf16(sr[sl], si[sl]);
+          for (int sl = 0; sl < NSL; ++sl) sY[(sl * TGD + row) * RW + c] = w[sl];
         }
       }
     }
@@ -724,7 +724,7 @@ __global__ void __launch_bounds__(TC_WARPS * 32, N == 16 ? (SAME ? 3 : 2) : 1)
       if (b >= GB::COUNT) break;  // uniform per warp
       int mt, nt;
       GB::at(b, mt, nt);
-      float d[6][4];
+      float d[6][4];  // D_u, u < NSL
 #pragma unroll
       for (int u = 0; u < 6; ++u)
 #pragma unroll
@@ -761,29 +761,38 @@ __global__ void __launch_bounds__(TC_WARPS * 32, N == 16 ? (SAME ? 3 : 2) : 1)
       }
     }
   }
-  gram_tc_write<N, true>(partials + (long long)blockIdx.x * N * N, gacc, 1.0, warp, lane);
+  gram_tc_write<N, true>(partials + (long long)blockIdx.x * n * n, gacc, 1.0, warp, lane, n);
 }
 
-template <int N, bool SAME>
-static cudaError_t launch_gram_tc_df(const void* X, const void* Y, int Vh, double2* partials,
-                                     int nblocks, Gate gate, cudaStream_t s) {
-  const size_t sm = (SAME ? 1 : 2) * (size_t)6 * TGD * (N + 4) * sizeof(uint32_t);
-  auto kern = k_gram_tc_df<N, SAME>;
+template <class S, int NP, bool SAME>
+static cudaError_t launch_gram_tc_df(const void* X, const void* Y, int N, int Vh,
+                                     double2* partials, int nblocks, Gate gate, cudaStream_t s) {
+  using E = typename S::elem;
+  const size_t sm =
+      (SAME ? 1 : 2) * (size_t)ozaki::SliceKind<S>::NSL * TGD * (NP + 4) * sizeof(uint32_t);
+  auto kern = k_gram_tc_df<S, NP, SAME>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  kern<<<nblocks, TC_WARPS * 32, sm, s>>>((const float4*)X, (const float4*)Y, Vh, partials, gate);
+  kern<<<nblocks, TC_WARPS * 32, sm, s>>>((const E*)X, (const E*)Y, N, Vh, partials, gate);
   return cudaGetLastError();
+}
+
+template <class S>
+static cudaError_t gram_split(const void* X, const void* Y, int N, int Vh, double2* partials,
+                              int nblocks, Gate gate, cudaStream_t s) {
+  if (N <= 16)
+    return X == Y ? launch_gram_tc_df<S, 16, true>(X, Y, N, Vh, partials, nblocks, gate, s)
+                  : launch_gram_tc_df<S, 16, false>(X, Y, N, Vh, partials, nblocks, gate, s);
+  return X == Y ? launch_gram_tc_df<S, 32, true>(X, Y, N, Vh, partials, nblocks, gate, s)
+                : launch_gram_tc_df<S, 32, false>(X, Y, N, Vh, partials, nblocks, gate, s);
 }
 
 // Hermitian Grams only (P^dag AP of the iteration)
 cudaError_t gram_partials_tc(FieldKind k, const void* X, const void* Y, int N, int Vh,
                              double2* partials, int nblocks, Gate gate, cudaStream_t s) {
-  if (k == FK_DF && N == 16)
-    return X == Y ? launch_gram_tc_df<16, true>(X, Y, Vh, partials, nblocks, gate, s)
-                  : launch_gram_tc_df<16, false>(X, Y, Vh, partials, nblocks, gate, s);
-  if (k == FK_DF && N == 32)
-    return X == Y ? launch_gram_tc_df<32, true>(X, Y, Vh, partials, nblocks, gate, s)
-                  : launch_gram_tc_df<32, false>(X, Y, Vh, partials, nblocks, gate, s);
+  if (!gram_tc_supported(k, N)) return cudaErrorInvalidValue;
+  if (k == FK_DF) return gram_split<StoreDF>(X, Y, N, Vh, partials, nblocks, gate, s);
+  if (k == FK_F32) return gram_split<StoreF32>(X, Y, N, Vh, partials, nblocks, gate, s);
   if (k == FK_H16) {
     if (N == 16) return launch_gram_tc<StoreH16, 16>(X, Y, Vh, partials, nblocks, gate, s);
     if (N == 32) return launch_gram_tc<StoreH16, 32>(X, Y, Vh, partials, nblocks, gate, s);
@@ -794,18 +803,22 @@ cudaError_t gram_partials_tc(FieldKind k, const void* X, const void* Y, int N, i
   return cudaErrorInvalidValue;
 }
 
-bool w_gram_tc_supported(FieldKind k, int N) {
+bool gram_tc_supported(FieldKind k, int N) {
+  if (k == FK_F32) return N > 8 && N <= 32;
   return (k == FK_DF || k == FK_H16 || k == FK_BF16) && (N == 16 || N == 32);
+}
+
+bool w_gram_tc_supported(FieldKind k, int N) {
+  return rows_tc_supported(k, N) || ((k == FK_H16 || k == FK_BF16) && (N == 16 || N == 32));
 }
 
 cudaError_t w_update_gram_tc(FieldKind k, void* Q, const void* AP, const double2* beta, int N,
                              int Vh, double2* partials, int nblocks, Gate gate, cudaStream_t s) {
-  if (k == FK_DF && (N == 16 || N == 32)) {
-    // double-float: W = Q - AP beta, then the Gram of the stored W (two passes)
-    cudaError_t e = w_update_tc_df(Q, AP, beta, N, Vh, gate, s);
-    if (e != cudaSuccess) return e;
-    return N == 16 ? launch_gram_tc_df<16, true>(Q, Q, Vh, partials, nblocks, gate, s)
-                   : launch_gram_tc_df<32, true>(Q, Q, Vh, partials, nblocks, gate, s);
+  if (rows_tc_supported(k, N)) {
+    // W = Q - AP beta, then the Gram of the stored W (two passes)
+    cudaError_t e = w_update_rows(k, Q, AP, beta, N, Vh, gate, s);
+    return e != cudaSuccess ? e
+                            : gram_partials(k, Q, Q, N, Vh, 1, partials, nblocks, gate, s, GR_TC);
   }
   if (k == FK_H16) {
     if (N == 16) return launch_w_gram_tc<StoreH16, 16>(Q, AP, beta, Vh, partials, nblocks, gate, s);
@@ -817,15 +830,20 @@ cudaError_t w_update_gram_tc(FieldKind k, void* Q, const void* AP, const double2
   return cudaErrorInvalidValue;
 }
 
+bool bcg_update_tracks(FieldKind sk, FieldKind xk, int N, int tile) {
+  return sk == FK_DF && (tile & UPD_TC) && bcg_update_tc_supported(sk, xk, N);
+}
+
 bool bcg_update_tc_supported(FieldKind sk, FieldKind xk, int N) {
-  if (sk == FK_DF) return xk == FK_DF && bcg_update_tc_df_supported(N);
+  if (sk == FK_DF || sk == FK_F32) return xk == FK_DF && rows_tc_supported(sk, N);
   return (sk == FK_H16 || sk == FK_BF16) && xk == FK_DF && (N == 16 || N == 32);
 }
 
 cudaError_t bcg_update_tc(FieldKind sk, void* Q, void* P, void* X, const double2* Sinv,
-                          const double2* BC, const double2* SH, int N, int Vh, Gate gate,
-                          cudaStream_t s) {
-  if (sk == FK_DF) return bcg_update_tc_df(Q, P, X, Sinv, BC, SH, N, Vh, gate, s);
+                          const double2* BC, const double2* SH, int N, int Vh, unsigned* pmax,
+                          Gate gate, cudaStream_t s) {
+  if (rows_tc_supported(sk, N))
+    return bcg_update_rows(sk, Q, P, X, Sinv, BC, SH, N, Vh, pmax, gate, s);
   if (sk == FK_H16) {
     if (N == 16) return launch_bcg_update_tc<StoreH16, 16>(Q, P, X, Sinv, BC, SH, Vh, gate, s);
     if (N == 32) return launch_bcg_update_tc<StoreH16, 32>(Q, P, X, Sinv, BC, SH, Vh, gate, s);

@@ -159,34 +159,40 @@ cudaError_t w_update_gram(FieldKind k, void* Q, const void* AP, const double2* b
 // thread and UPD_X_GLOBAL for the old X read from global memory (not staged)
 static constexpr int UPD_TWO_ROWS = 64;
 static constexpr int UPD_X_GLOBAL = 128;
-// tile | UPD_TC: the tensor-core form (16-bit kinds with N = 16 or 32, the
-// double-float kind with N = 16; the CUDA-core kernel otherwise)
+// tile | UPD_TC: the tensor-core form (16-bit kinds with N = 16 or 32,
+// double-float and FP32 with 3 <= N <= 32; the CUDA-core kernel otherwise)
 static constexpr int UPD_TC = 256;
 // tile | WG_TC for w_update_gram: the tensor-core fused W + Gram (16-bit
-// kinds, N = 16 or 32; the FP32-pipe kernel otherwise)
+// kinds, N = 16 or 32), or the tensor-core W update and a Gram of the result
+// (double-float and FP32, 3 <= N <= 32; the FP32-pipe kernel otherwise)
 static constexpr int WG_TC = 256;
-// tile | GR_TC for gram_partials: the tensor-core Gram (Hermitian Grams of
-// the 16-bit kinds, N = 16 or 32; the FP32-pipe kernel otherwise)
+// tile | GR_TC for gram_partials: the tensor-core Gram (Hermitian Grams of the
+// pairs of gram_tc_supported; the FP32-pipe kernel otherwise)
 static constexpr int GR_TC = 256;
 // Q <- W Sinv ; X += P BC ; P <- Q + P SH unless st->ru_pending
+// pmax (bcg_update_tracks only, else null): N words that receive the maxima of the
+// new P's columns as the digit stencil counts them (zeroed by the caller)
 cudaError_t bcg_update(FieldKind sk, FieldKind xk, void* Q, void* P, void* X, const double2* Sinv,
                        const double2* BC, const double2* SH, int N, int Vh, Gate gate,
-                       cudaStream_t s, int tile = 0);
-// the tensor-core fused update of the double-float kind (blas_tc_df.cu,
-// exact split bf16 products), N = 16
-bool bcg_update_tc_df_supported(int N);
-cudaError_t bcg_update_tc_df(void* Q, void* P, void* X, const double2* Sinv, const double2* BC,
-                             const double2* SH, int N, int Vh, Gate gate, cudaStream_t s);
-// W = Q - AP beta over Q for the double-float kind on the tensor cores, N = 16
-cudaError_t w_update_tc_df(void* Q, const void* AP, const double2* beta, int N, int Vh, Gate gate,
-                           cudaStream_t s);
+                       cudaStream_t s, int tile = 0, unsigned* pmax = nullptr);
+bool bcg_update_tracks(FieldKind sk, FieldKind xk, int N, int tile);
+// the tensor-core fused update and W = Q - AP beta of the double-float and the
+// FP32 kind (blas_rows.cu, exact split bf16 products), 3 <= N <= 32; X is
+// double-float
+bool rows_tc_supported(FieldKind k, int N);
+cudaError_t bcg_update_rows(FieldKind k, void* Q, void* P, void* X, const double2* Sinv,
+                            const double2* BC, const double2* SH, int N, int Vh, unsigned* pmax,
+                            Gate gate, cudaStream_t s);
+cudaError_t w_update_rows(FieldKind k, void* Q, const void* AP, const double2* beta, int N, int Vh,
+                          Gate gate, cudaStream_t s);
 // the tensor-core fused update (blas_tc.cu): supported (kind, N) pairs
 bool bcg_update_tc_supported(FieldKind sk, FieldKind xk, int N);
 cudaError_t bcg_update_tc(FieldKind sk, void* Q, void* P, void* X, const double2* Sinv,
-                          const double2* BC, const double2* SH, int N, int Vh, Gate gate,
-                          cudaStream_t s);
+                          const double2* BC, const double2* SH, int N, int Vh, unsigned* pmax,
+                          Gate gate, cudaStream_t s);
 bool w_gram_tc_supported(FieldKind k, int N);
-// Hermitian K = X^dag Y on the tensor cores (the pairs of w_gram_tc_supported)
+// Hermitian K = X^dag Y on the tensor cores
+bool gram_tc_supported(FieldKind k, int N);
 cudaError_t gram_partials_tc(FieldKind k, const void* X, const void* Y, int N, int Vh,
                              double2* partials, int nblocks, Gate gate, cudaStream_t s);
 cudaError_t w_update_gram_tc(FieldKind k, void* Q, const void* AP, const double2* beta, int N,

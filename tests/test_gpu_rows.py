@@ -1,0 +1,46 @@
+"""GPU tests of the tensor-core block BLAS of the double-float and FP32 kinds (update,
+W update, Gram) at widths around its paddings of 8, 16 and 32 columns, through whole
+solves with each kernel forced by the tuning cache."""
+import json
+
+import numpy as np
+import pytest
+
+import hisq_inputs as hi
+from oracle import hisq
+from tests import gpu_helpers as gh
+
+pytestmark = pytest.mark.gpu
+
+KIND = {"f64": 0, "mixed_f32": 1}
+UPD, WGRAM, GRAM = 1 << 24, 1 << 25, 1 << 26
+
+
+@pytest.mark.parametrize("prec", list(KIND))
+@pytest.mark.parametrize("N", [3, 8, 9, 15, 17, 31, 32])
+def test_forced_kernels_converge(tmp_path, prec, N):
+    """Each kernel alone and all together meet tol on the oracle's residual in as many
+    iterations as the CUDA-core kernels (one more or less for double-float, a tenth for
+    FP32); 6 x 4 x 6 x 10 has 2160 rows, a whole number of 16-row tiles, 33 and 3/4
+    tiles of 64."""
+    torch = gh.torch_mod()
+    dims, mass, tol = (6, 4, 6, 10), 0.1, 1e-11
+    dev = torch.cuda.get_device_name().replace(" ", "_")
+    b = hi.gaussian_sources(dims, N, seed=91 + N)
+    iters = {}
+    for name, flags in (("cores", 0), ("upd", UPD), ("wgram", WGRAM), ("gram", GRAM),
+                        ("all", UPD | WGRAM | GRAM)):
+        path = tmp_path / f"{name}.json"
+        path.write_text(json.dumps({f"blas/6.4.6.10/kind{KIND[prec]}/N{N}/{dev}":
+                                    8 | (8 << 8) | (8 << 16) | flags}))
+        s, fat, lng = gh.make_solver(dims, mass, prec=prec, seed=90, max_rhs=N)
+        s.set_tune_cache(path)
+        X, info = s.solve(b, tol=tol)
+        assert info["status"] == 0, name
+        X = gh.to_np(X)
+        r = (b - hisq.apply_A(dims, fat, lng, mass, X)).reshape(N, -1)
+        rel = np.linalg.norm(r, axis=1) / np.linalg.norm(b.reshape(N, -1), axis=1)
+        assert rel.max() <= tol * 1.01, (name, rel)
+        iters[name] = info["iters"]
+    for name in iters:
+        assert abs(iters[name] - iters["cores"]) <= (1 if prec == "f64" else iters["cores"] // 10), iters
