@@ -1156,12 +1156,20 @@ void blockcg_destroy(blockcg_t h) {
   delete h;
 }
 
+// Whether the gauge storage holds the digit stencil's links.  The forms with an
+// FP32 or 16-bit iteration use them in the reliable updates alone, for FP64 from
+// Vh N = 2^18 (fx_allowed), and N is at most 64: a smaller lattice does without
+// their 2.5 KB per site and parity, and its updates keep the CUDA-core kernels.
+static bool fx_stored(const blockcg_ctx* h) {
+  return h->sloppy == FK_DF || h->sloppy == FK_F64 || h->g.Vh >= (1 << 18) / 64;
+}
+
 size_t blockcg_gauge_bytes(blockcg_t h) {
   if (!h) return 0;
   size_t b = up(links_bytes(h->fine, h->g));
   if (h->sloppy != h->fine) b += up(links_bytes(h->sloppy, h->g, h->p.link_recon));
   if (h->ru != h->fine && h->ru != h->sloppy) b += up(links_bytes(h->ru, h->g));
-  b += up(fx_links_bytes(h->g));
+  if (fx_stored(h)) b += up(fx_links_bytes(h->g));
   if (h->p.link_recon) b += ALIGN;  // scratch of the link check
   return b;
 }
@@ -1196,7 +1204,7 @@ blockcg_status blockcg_load_gauge(blockcg_t h, const void* fat, const void* lng,
   h->gauge = storage;
   h->gauge_bytes = storage_bytes;
   // [FP64 links][iteration links, if another kind][reliable-update links, if
-  // a third kind][the digit stencil's links]
+  // a third kind][the digit stencil's links, fx_stored]
   char* next = (char*)storage + up(links_bytes(h->fine, h->g));
   h->links_fine = storage;
   h->links_sloppy = storage;
@@ -1214,8 +1222,11 @@ blockcg_status blockcg_load_gauge(blockcg_t h, const void* fat, const void* lng,
     CK(pack_links(h->ru, (const double2*)fat, (const double2*)lng, h->links_ru, h->g,
                   h->p.antiperiodic_t, 0, h->stream));
   if (h->ru != h->fine && h->ru != h->sloppy) next += up(links_bytes(h->ru, h->g));
-  CK(fx_pack_links(h->links_fine, next, h->g, h->stream));
-  h->g.fx_links = next;
+  h->g.fx_links = nullptr;
+  if (fx_stored(h)) {
+    CK(fx_pack_links(h->links_fine, next, h->g, h->stream));
+    h->g.fx_links = next;
+  }
   h->gauge_loaded = true;
   return BLOCKCG_OK;
 }
