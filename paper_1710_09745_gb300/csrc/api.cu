@@ -684,6 +684,18 @@ double cheap_ru_above(const blockcg_ctx* h) {
   return (h->sloppy == FK_H16 || h->sloppy == FK_BF16) ? 1e2 : 1e4;
 }
 
+// Whether the iteration's update leaves the new P's column maxima for the digit
+// stencil's first half; whoever else writes P, or runs another digit stencil,
+// takes them again (prime_pmax).
+bool tracks_pmax(const blockcg_ctx* h, int N) {
+  return h->sloppy == FK_DF && (cached_R(h, FK_DF, N) & DSLASH_TC) && dslash_fx_supported(h->g, N) &&
+         bcg_update_tracks(FK_DF, h->upd, N, cached_tiles(h, FK_DF, N).upd);
+}
+blockcg_status prime_pmax(blockcg_ctx* h, const Ws& w, int N, Gate gate) {
+  if (tracks_pmax(h, N)) TL(TC_STREAM, fx_column_max(w.P, h->g, N, gate, h->stream));
+  return BLOCKCG_OK;
+}
+
 // A reliable update (Algorithm 3) gated by `gate`: with a cheaper kind, two
 // residual blocks gated on this iteration's residual (GATE_RU_CHEAP /
 // GATE_RU_FINE, exactly one of them runs); otherwise the FP64 one.
@@ -723,7 +735,7 @@ blockcg_status verify_fp64(blockcg_ctx* h, const Ws& w, int N, double tol) {
   TL(TC_GRAM, gram_partials(FK_F64, w.R, w.R, N, h->g.Vh, 1, w.partials, w.nblocks, g0, s));
   TL(TC_GRAM, gram_reduce(w.partials, w.nblocks, N, 1, mat(w, M_K, N), g0, s));
   TL(TC_DENSE, dense_verify(mat(w, M_K, N), w.bnorm, w.tres, tol, N, w.st, s));
-  return BLOCKCG_OK;
+  return prime_pmax(h, w, N, g0);  // should the iteration go on
 }
 
 // one iteration of Algorithm 1 up to the decision on a reliable update
@@ -733,8 +745,9 @@ blockcg_status iterate_core(blockcg_ctx* h, const Ws& w, int N, double tol, Loop
   double m2 = h->mass * h->mass;
   cudaStream_t s = h->stream;
   FieldKind k = h->sloppy;
-  SL(0, dslash(k, R | DSLASH_FIRST, EPI_NONE, h->links_sloppy, w.P, w.Ts, nullptr, nullptr, 0.0, h->g,
-               1, N, ga, s));
+  const bool maxed = tracks_pmax(h, N);
+  SL(0, dslash(k, R | DSLASH_FIRST | (maxed ? DSLASH_MAXED : 0), EPI_NONE, h->links_sloppy, w.P, w.Ts,
+               nullptr, nullptr, 0.0, h->g, 1, N, ga, s));
   SL(0, dslash(k, R | DSLASH_SECOND, EPI_NORMAL, h->links_sloppy, w.Ts, w.AP, w.P, nullptr, m2, h->g,
                0, N, ga, s));
   const BlasTiles bt = cached_tiles(h, k, N);
@@ -749,14 +762,20 @@ blockcg_status iterate_core(blockcg_ctx* h, const Ws& w, int N, double tol, Loop
   TL(TC_DENSE, dense_qr_step(mat(w, M_G, N), mat(w, M_C, N), mat(w, M_CPREV, N), mat(w, M_SINV, N),
                    mat(w, M_SH, N), w.bnorm, qp, N, w.st, ga, ctl, s));
   TL(TC_STREAM, bcg_update(k, h->upd, w.Q, w.P, w.X, mat(w, M_SINV, N), mat(w, M_BC, N), mat(w, M_SH, N), N,
-                h->g.Vh, ga, s, bt.upd));
+                h->g.Vh, ga, s, bt.upd, maxed ? h->g.fx_ctl : nullptr));
   return BLOCKCG_OK;
+}
+
+// the pending reliable update of an iteration
+blockcg_status update_block(blockcg_ctx* h, const Ws& w, int N, double tol, Gate gate, LoopCtl ctl) {
+  blockcg_status rc = restart_block(h, w, N, tol, 0, gate, ctl);
+  return rc ? rc : prime_pmax(h, w, N, gate);
 }
 
 // the same with the gated reliable update, as the host enqueues it
 blockcg_status iterate_block(blockcg_ctx* h, const Ws& w, int N, double tol) {
   blockcg_status rc = iterate_core(h, w, N, tol, LoopCtl{});
-  return rc ? rc : restart_block(h, w, N, tol, 0, Gate{w.st, GATE_RU, 0.0, true});
+  return rc ? rc : update_block(h, w, N, tol, Gate{w.st, GATE_RU, 0.0, true}, LoopCtl{});
 }
 
 blockcg_status status_to_result(blockcg_ctx* h, const SolverStatus& st) {
@@ -907,7 +926,7 @@ blockcg_status build_loop(blockcg_ctx* h, const Ws& w, int N, double tol, int un
   const long long l1 = h->launches;
   for (int i = 0; i < unroll; ++i) {
     rc = capture_into(h, update[i], [&] {
-      return restart_block(h, w, N, tol, 0, Gate{w.st, GATE_RU, 0.0, false}, ctls[i]);
+      return update_block(h, w, N, tol, Gate{w.st, GATE_RU, 0.0, false}, ctls[i]);
     });
     if (rc) return rc;
   }
@@ -1359,6 +1378,8 @@ blockcg_status blockcg_solve(blockcg_t h, const void* B, void* X, int n_rhs, dou
   rc = solve_begin(h, w, B, X, N, tol);
   if (rc) return rc;
   tune_block(h, w, N);
+  rc = prime_pmax(h, w, N, Gate{nullptr, GATE_ALWAYS});
+  if (rc) return rc;
   SolverStatus hs;
   memset(&hs, 0, sizeof(hs));
   // a caller that profiles or polls gets the host-driven loop
@@ -1911,6 +1932,7 @@ blockcg_status blockcg_batch_solve(blockcg_batch_t b, const void* const* B, void
     Ws w = carve(h, N[p], h->ws);
     long long l0 = h->launches;
     blockcg_status rc = solve_begin(h, w, B[p], X[p], N[p], tol);
+    if (!rc) rc = prime_pmax(h, w, N[p], Gate{nullptr, GATE_ALWAYS});
     if (rc) return pfail(b, p, rc);
     launches += h->launches - l0;
     BK(cudaEventRecord(b->done_ev[p], b->streams[p]));

@@ -104,10 +104,15 @@ static constexpr int DSLASH_TC = 0x2000;
 // the other kernels ignore both flags)
 static constexpr int DSLASH_FIRST = 0x4000;
 static constexpr int DSLASH_SECOND = 0x8000;
+// a first half whose input's column maxima are already in the control words
+// (bcg_update's pmax, fx_column_max)
+static constexpr int DSLASH_MAXED = 0x20000;
 // R | DSLASH_SPLIT, R = 4 or 16 lanes per output: the hop-split kernel
 // (full links, 32- and 64-bit kinds; an autotuner candidate on small problems)
 static constexpr int DSLASH_SPLIT = 0x10000;
 bool dslash_fx_supported(const Geom& g, int N);
+// the column maxima of a double-float block on even sites into the control words
+cudaError_t fx_column_max(const void* f, const Geom& g, int N, Gate gate, cudaStream_t s);
 size_t fx_links_bytes(const Geom& g);
 size_t fx_digit_bytes(const Geom& g, int N);
 // the digit stencil's links from the packed FP64 ones
@@ -171,7 +176,7 @@ static constexpr int WG_TC = 256;
 static constexpr int GR_TC = 256;
 // Q <- W Sinv ; X += P BC ; P <- Q + P SH unless st->ru_pending
 // pmax (bcg_update_tracks only, else null): N words that receive the maxima of the
-// new P's columns as the digit stencil counts them (zeroed by the caller)
+// new P's columns as fx_column_max counts them (zeroed by the caller)
 cudaError_t bcg_update(FieldKind sk, FieldKind xk, void* Q, void* P, void* X, const double2* Sinv,
                        const double2* BC, const double2* SH, int N, int Vh, Gate gate,
                        cudaStream_t s, int tile = 0, unsigned* pmax = nullptr);

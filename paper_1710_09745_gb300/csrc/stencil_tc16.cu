@@ -3,7 +3,7 @@
 // (Sec. 6.2) as per-site products on mma.sync with FP32 accumulation.
 //
 // The stored 16-bit spinors and links are exact MMA operands, so nothing is
-// split (compare stencil_tc.cu): with the 16 hops and 3 colours as a K index
+// split (compare stencil_fx.cuh): with the 16 hops and 3 colours as a K index
 // of 96 reals, one warp computes one site's out^T = Psi^T U^T, A = the
 // gathered neighbour spinors (M = 16 right-hand sides per tile; a stored
 // (re, im) pair is one A register as it is), B = the site's hop matrices in
@@ -47,7 +47,7 @@ struct Tc16Mma<StoreBF16> {
 
 }  // namespace
 
-// Lane = (gq, tig) as in k_dslash_tc: rows gq, gq + 8 of A (right-hand
+// Lane = (gq, tig) as in k_dslash_fx: rows gq, gq + 8 of A (right-hand
 // sides), complex K entries tig and tig + 4 of each 8-entry chunk, B column
 // gq, outputs (colour tig, right-hand sides gq and gq + 8).
 template <class S, int EPI, int MT>

@@ -44,3 +44,28 @@ def test_forced_kernels_converge(tmp_path, prec, N):
         iters[name] = info["iters"]
     for name in iters:
         assert abs(iters[name] - iters["cores"]) <= (1 if prec == "f64" else iters["cores"] // 10), iters
+
+
+@pytest.mark.parametrize("N", [3, 8, 16, 24])
+def test_update_leaves_the_column_maxima(tmp_path, N):
+    """The digit stencil scales P's columns by the maxima that the tensor-core update
+    leaves: the solve takes the iterations that it takes when the stencil finds them
+    itself (the CUDA-core update), through reliable updates, and meets tol."""
+    torch = gh.torch_mod()
+    dims, mass, tol = (6, 4, 6, 10), 0.1, 1e-11
+    dev = torch.cuda.get_device_name().replace(" ", "_")
+    b = hi.gaussian_sources(dims, N, seed=71 + N)
+    iters = []
+    for flags in (0, UPD):
+        path = tmp_path / f"{flags}.json"
+        path.write_text(json.dumps({f"blas/6.4.6.10/kind0/N{N}/{dev}":
+                                    8 | (8 << 8) | (8 << 16) | flags}))
+        s, fat, lng = gh.make_solver(dims, mass, seed=70, max_rhs=N, dslash_variant=8192 + 1)
+        s.set_tune_cache(path)
+        X, info = s.solve(b, tol=tol)
+        assert info["status"] == 0 and info["reliable_updates"] >= 1
+        r = (b - hisq.apply_A(dims, fat, lng, mass, gh.to_np(X))).reshape(N, -1)
+        rel = np.linalg.norm(r, axis=1) / np.linalg.norm(b.reshape(N, -1), axis=1)
+        assert rel.max() <= tol * 1.01, (flags, rel)
+        iters.append(info["iters"])
+    assert abs(iters[0] - iters[1]) <= 1, iters
