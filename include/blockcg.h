@@ -393,24 +393,23 @@ blockcg_status blockcg_block_cdot_noalloc(const void* X, const void* Y, int n_rh
  * per-iteration kernel sequence of blockcg_solve (Algorithm 1 with the gated
  * reliable update of Algorithm 3) for every problem runs on a stream of its
  * own, so small lattices that cannot fill the GPU alone run side by side.
- * With BLOCKCG_BATCH_GRAPH, one chunk of iterations of every active problem
- * is captured once into a single CUDA graph and replayed until each problem
- * has converged, failed or reached its max_iter (the graph is captured again
- * when the set of active problems changes).  The stencil autotuner runs once
+ * With BLOCKCG_BATCH_GRAPH, the loops of all problems are captured once into
+ * a single CUDA graph; each runs on the device until its problem has
+ * converged, failed or reached its max_iter.  The stencil autotuner runs once
  * per (lattice, storage kind, N) and its choice is shared by the batch.
  * Results are the same as blockcg_solve on each handle.  The paper solves
  * one block at a time; batching many problems is this library's extension. */
 typedef struct blockcg_batch* blockcg_batch_t;
 
 #define BLOCKCG_BATCH_MAX 4096
-#define BLOCKCG_BATCH_GRAPH 1 /* flags bit: replay a captured CUDA graph */
+#define BLOCKCG_BATCH_GRAPH 1 /* flags bit: one captured CUDA graph loops on the device */
 /* flags bits 8..15: iterations per device-loop trip with BLOCKCG_BATCH_GRAPH
  * (0: chosen from the problem's size; at most 16) */
 #define BLOCKCG_BATCH_TRIP_SHIFT 8
 
 typedef struct {
   double ms_total;         /* device time of the whole batch (CUDA events) */
-  int chunk;               /* iterations per replay (min of the problems' check_every) */
+  int chunk;               /* iterations per device-loop trip, or between host polls */
   long long graph_replays; /* graph launches (0 without BLOCKCG_BATCH_GRAPH) */
   long long graph_captures;
   long long graph_nodes;   /* nodes of the last captured graph */
