@@ -59,6 +59,8 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 // slices, kept products (s + t < NU) and their sum by storage kind
 struct KindDF : SliceKind<StoreDF> {  // six slices, 21 products
   using Store = StoreDF;
+  using In = float4;  // an entry of the rows that are multiplied
+  static __device__ __forceinline__ In in_zero() { return zero(); }
   static constexpr int NU = 6;
   static __device__ __forceinline__ dfacc sum(const float (&a)[NU][4], int i) {
     float h = a[0][i], l = __fadd_rn(a[5][i], a[4][i]);
@@ -68,8 +70,14 @@ struct KindDF : SliceKind<StoreDF> {  // six slices, 21 products
     return {h, l};
   }
 };
+struct KindF64 : KindDF {  // the same of FP64 rows (QROWS), scaled before they are rounded
+  using In = double2;
+  static __device__ __forceinline__ In in_zero() { return make_double2(0.0, 0.0); }
+};
 struct KindDF7 : SliceKind<StoreDF> {  // seven slices, 28 products
   using Store = StoreDF;
+  using In = float4;
+  static __device__ __forceinline__ In in_zero() { return zero(); }
   static constexpr int NSL = 7, NU = 7;
   static __device__ __forceinline__ void slices(float4 v, float sc, uint32_t (&w)[NSL]) {
     float re[7], im[7];
@@ -88,6 +96,8 @@ struct KindDF7 : SliceKind<StoreDF> {  // seven slices, 28 products
 };
 struct KindF32 : SliceKind<StoreF32> {  // four slices, 10 products
   using Store = StoreF32;
+  using In = float2;
+  static __device__ __forceinline__ In in_zero() { return zero(); }
   static constexpr int NU = 4;
   static __device__ __forceinline__ dfacc sum(const float (&a)[NU][4], int i) {
     float h = a[0][i], l = __fadd_rn(a[3][i], a[2][i]);
@@ -96,37 +106,45 @@ struct KindF32 : SliceKind<StoreF32> {  // four slices, 10 products
   }
 };
 
-template <class K, int NP, bool WMODE>
+// what a launch computes (the matrix passed as Sinv but in UPDATE)
+enum RowsMode {
+  UPDATE,  // Q = W S^-1 (W in Q), X += P (beta C), P = Q + P S^dag
+  WROWS,   // Q = Q - P beta
+  QROWS,   // Q = P C, C upper triangular; Q in FP32, P in the kind's In
+  PROWS,   // P = Q + P S
+};
+
+template <class K, int NP, int MODE>
 struct RtGeom {
   static constexpr int KS = NP / 8;  // k steps of 16 reals (8 complex numbers)
   static constexpr int NT = NP / 4;  // output tiles of 8 reals (4 complex columns)
-  static constexpr int NM = WMODE ? 1 : 3;
+  static constexpr int NM = MODE != UPDATE ? 1 : 3;
   static constexpr int FR = KS * NT * 32;
   static constexpr size_t smem = (size_t)NM * K::NSL * FR * sizeof(uint2);
   // warps per SM: 12 of up to 168 registers in one CTA; 16 of 128 where the
   // slices leave room (24^4, FP32, N = 32 update: 325 us against 349; 32^4,
   // double-float, N = 16: 640 against 690, and as two CTAs, which start up apart)
   static constexpr int threads =
-      std::is_same<K, KindF32>::value && NP == 32 ? 512 : std::is_same<K, KindDF>::value && NP == 16 ? 256 : 384;
+      std::is_same<K, KindF32>::value && NP == 32 ? 512 : std::is_base_of<KindDF, K>::value && NP == 16 ? 256 : 384;
   static constexpr int ctas = threads == 256 ? 2 : 1;
   // the slices of W and P together: where they leave room (double-float, N = 16:
   // 830 us together, 682 in turn; N = 8 30 against 32, FP32 N = 16 40 against 44)
-  static constexpr bool both = !WMODE && (NP == 8 || (NP == 16 && std::is_same<K, KindF32>::value));
+  static constexpr bool both = MODE == UPDATE && (NP == 8 || (NP == 16 && std::is_same<K, KindF32>::value));
 };
 
 }  // namespace
 
-// WMODE: the W update of Algorithm 1 instead, W = Q - AP beta over Q (AP
-// passed as P, beta as Sinv; one full coefficient matrix)
-template <class K, int NP, bool WMODE>
-__global__ void __launch_bounds__((RtGeom<K, NP, WMODE>::threads), (RtGeom<K, NP, WMODE>::ctas))
-    k_rows_tc(typename K::Store::elem* __restrict__ Q, typename K::Store::elem* __restrict__ P,
-              float4* __restrict__ X, const double2* __restrict__ Sinv,
+template <class K, int NP, int MODE>
+__global__ void __launch_bounds__((RtGeom<K, NP, MODE>::threads), (RtGeom<K, NP, MODE>::ctas))
+    k_rows_tc(std::conditional_t<MODE == QROWS, float2, typename K::Store::elem>* __restrict__ Q,
+              typename K::In* __restrict__ P, float4* __restrict__ X, const double2* __restrict__ Sinv,
               const double2* __restrict__ BC, const double2* __restrict__ SH, int N, int Vh,
               unsigned* __restrict__ pmax, Gate gate) {
   using S = typename K::Store;
-  using G = RtGeom<K, NP, WMODE>;
+  using G = RtGeom<K, NP, MODE>;
   using E = typename S::elem;
+  using In = typename K::In;
+  constexpr bool WMODE = MODE != UPDATE;  // one matrix
   constexpr bool DF = std::is_same<S, StoreDF>::value;
   constexpr int KS = G::KS, NT = G::NT, NM = G::NM, FR = G::FR, NSL = K::NSL, NU = K::NU;
   constexpr bool BOTH = G::both;
@@ -139,7 +157,7 @@ __global__ void __launch_bounds__((RtGeom<K, NP, WMODE>::threads), (RtGeom<K, NP
   const bool keepP = gate.st != nullptr && ((const volatile SolverStatus*)gate.st)->ru_pending;
   auto Ms = [&](int m) { return m == 0 ? Sinv : m == 1 ? BC : SH; };
   auto in_pattern = [&](int m, int i, int j) {
-    return i < N && j < N && (WMODE || rt_in_pattern(m, i, j));
+    return i < N && j < N && (MODE == WROWS || MODE == PROWS || rt_in_pattern(m, i, j));
   };
   if (threadIdx.x < NP) sM[threadIdx.x] = 0u;
   for (int c = threadIdx.x; c < NM * NP; c += RT_THREADS) {
@@ -152,7 +170,8 @@ __global__ void __launch_bounds__((RtGeom<K, NP, WMODE>::threads), (RtGeom<K, NP
     }
     int e = 0;
     if (mx > 0.0 && mx < 1e300) frexp(mx, &e);  // mx in [2^(e-1), 2^e)
-    sE[c] = e < -120 ? -120 : e > 120 ? 120 : e;
+    constexpr int EMAX = MODE == QROWS ? 1000 : 120;
+    sE[c] = e < -EMAX ? -EMAX : e > EMAX ? EMAX : e;
   }
   __syncthreads();
   // B fragments: k step ks, lane (g, t): b.x holds rows (re, im) of input
@@ -197,26 +216,26 @@ __global__ void __launch_bounds__((RtGeom<K, NP, WMODE>::threads), (RtGeom<K, NP
   for (long long tile = (long long)blockIdx.x * RT_WARPS + warp; tile < ntiles; tile += stride) {
     const long long ra = tile * 16 + g, rb = ra + 8;
     const bool va = ra < nrows, vb = rb < nrows;
-    auto prefetch = [&](const E* f, long long r) {
+    auto prefetch = [&](const In* f, long long r) {
       if (r < nrows && 4 * t < N) prefetch_l2(f + r * N + 4 * t);
     };
+    prefetch(P, ra + 16 * stride);
+    prefetch(P, rb + 16 * stride);
     if constexpr (!WMODE) {
-      prefetch(reinterpret_cast<const E*>(P), ra + 16 * stride);
-      prefetch(reinterpret_cast<const E*>(P), rb + 16 * stride);
+      prefetch((const In*)Q, ra + 16 * stride);
+      prefetch((const In*)Q, rb + 16 * stride);
     }
-    prefetch(WMODE ? P : Q, ra + 16 * stride);
-    prefetch(WMODE ? P : Q, rb + 16 * stride);
     // this thread's entries of rows ra, rb: v[ks][0..3] = (ra, c0), (rb, c0),
     // (ra, c0 + 1), (rb, c0 + 1), c0 = 8 ks + 2 t
-    auto load = [&](const E* src, E (&v)[KS][4]) {
+    auto load = [&](const In* src, In (&v)[KS][4]) {
 #pragma unroll
       for (int ks = 0; ks < KS; ++ks) {
         const int c0 = 8 * ks + 2 * t;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const bool ok = h ? vb : va;
-          const E* p = src + (h ? rb : ra) * N + c0;
-          v[ks][h] = v[ks][2 + h] = K::zero();
+          const In* p = src + (h ? rb : ra) * N + c0;
+          v[ks][h] = v[ks][2 + h] = K::in_zero();
           if constexpr (std::is_same<S, StoreF32>::value) {
             if (pairs) {
               if (ok && c0 < N) {
@@ -234,29 +253,56 @@ __global__ void __launch_bounds__((RtGeom<K, NP, WMODE>::threads), (RtGeom<K, NP
     };
     // A fragments of all slices, and the row exponents (the four threads t of
     // a row hold its N entries)
-    auto split = [&](const E (&v)[KS][4], uint32_t (&a)[KS][NSL][4], int (&er)[2]) {
-      float mx[2] = {0.f, 0.f};
+    auto split = [&](const In (&v)[KS][4], uint32_t (&a)[KS][NSL][4], int (&er)[2]) {
+      if constexpr (std::is_same<In, double2>::value) {
+        unsigned mx[2] = {0u, 0u};  // high words
+        auto high = [](double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; };
 #pragma unroll
-      for (int ks = 0; ks < KS; ++ks)
+        for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) mx[i & 1] = fmaxf(mx[i & 1], K::mag(v[ks][i]));
-      float sc[2];
+          for (int i = 0; i < 4; ++i) mx[i & 1] = max(mx[i & 1], max(high(v[ks][i].x), high(v[ks][i].y)));
+        double sc[2];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
-        mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
-        er[h] = pow2_above(__float_as_uint(mx[h]));
-        sc[h] = exp2i(-er[h]);
-      }
-#pragma unroll
-      for (int ks = 0; ks < KS; ++ks)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          uint32_t w[NSL];
-          K::slices(v[ks][i], sc[i & 1], w);
-#pragma unroll
-          for (int s = 0; s < NSL; ++s) a[ks][s][i] = w[s];
+        for (int h = 0; h < 2; ++h) {
+          mx[h] = max(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
+          mx[h] = max(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
+          er[h] = min(max((int)(mx[h] >> 20) - 1022, -1000), 1000);  // |row| < 2^er
+          sc[h] = __hiloint2double((1023 - er[h]) << 20, 0);
         }
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const double2 z = make_double2(v[ks][i].x * sc[i & 1], v[ks][i].y * sc[i & 1]);
+            uint32_t w[NSL];
+            K::slices(StoreDF::from_double2(z), 1.f, w);
+#pragma unroll
+            for (int s = 0; s < NSL; ++s) a[ks][s][i] = w[s];
+          }
+      } else {
+        float mx[2] = {0.f, 0.f};
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) mx[i & 1] = fmaxf(mx[i & 1], K::mag(v[ks][i]));
+        float sc[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
+          mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
+          er[h] = pow2_above(__float_as_uint(mx[h]));
+          sc[h] = exp2i(-er[h]);
+        }
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            uint32_t w[NSL];
+            K::slices(v[ks][i], sc[i & 1], w);
+#pragma unroll
+            for (int s = 0; s < NSL; ++s) a[ks][s][i] = w[s];
+          }
+      }
     };
     // rows times coefficient matrix m, output tile nt; k steps kf .. kl
     auto product = [&](int m, int nt, const uint32_t (&a)[KS][NSL][4], float (&acc)[NU][4], int kf,
@@ -279,6 +325,11 @@ __global__ void __launch_bounds__((RtGeom<K, NP, WMODE>::threads), (RtGeom<K, NP
     };
     // (re, im) of output (row h, complex column 4 nt + t)
     auto value = [&](const float (&acc)[NU][4], int h, int er, int ej) {
+      if constexpr (MODE == QROWS) {  // the exponents are large and of opposite sign
+        const int e = min(max(er + ej, -240), 240);
+        er = e / 2;
+        ej = e - er;
+      }
       const float fa = exp2i(er), fb = exp2i(ej);
       cpx<dfacc> v{K::sum(acc, 2 * h), K::sum(acc, 2 * h + 1)};
       v.re = {__fmul_rn(__fmul_rn(v.re.s, fa), fb), __fmul_rn(__fmul_rn(v.re.e, fa), fb)};
@@ -316,7 +367,7 @@ __global__ void __launch_bounds__((RtGeom<K, NP, WMODE>::threads), (RtGeom<K, NP
       uint32_t a[KS][NSL][4];
       int er[2];
       {
-        E v[KS][4];
+        In v[KS][4];
         load(P, v);
         split(v, a, er);
       }
@@ -324,14 +375,24 @@ __global__ void __launch_bounds__((RtGeom<K, NP, WMODE>::threads), (RtGeom<K, NP
       for (int nt = 0; nt < NT; ++nt) {
         const int j = 4 * nt + t;
         E q[2];
+        if constexpr (MODE != QROWS) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            q[h] = (h ? vb : va) && j < N ? Q[(h ? rb : ra) * N + j] : K::zero();
+        }
+        product(0, nt, a, acc, 0, MODE == QROWS ? k_last_upper(nt) : KS - 1);
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-          q[h] = (h ? vb : va) && j < N ? Q[(h ? rb : ra) * N + j] : K::zero();
-        product(0, nt, a, acc, 0, KS - 1);
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-          if ((h ? vb : va) && j < N)
-            put(Q + (h ? rb : ra) * N + j, plus(as_df(q[h]), value(acc, h, er[h], sE[j]), -1.f));
+          if ((h ? vb : va) && j < N) {
+            const long long o = (h ? rb : ra) * N + j;
+            const cpx<df> v = value(acc, h, er[h], sE[j]);
+            if constexpr (MODE == WROWS)
+              put(Q + o, plus(as_df(q[h]), v, -1.f));
+            else if constexpr (MODE == PROWS)
+              put(P + o, plus(as_df(q[h]), v, 1.f));
+            else
+              Q[o] = make_float2(v.re.hi, v.im.hi);
+          }
       }
     } else if constexpr (BOTH) {
       uint32_t aw[KS][NSL][4], ap[KS][NSL][4];
@@ -447,15 +508,14 @@ bool rows_tc_supported(FieldKind k, int N) {
   return (k == FK_DF || k == FK_F32) && N >= 3 && N <= 32;
 }
 
-template <class K, int NP, bool WMODE>
+template <class K, int NP, int MODE>
 static cudaError_t launch_rows(void* Q, void* P, void* X, const double2* Sinv, const double2* BC,
                                const double2* SH, int N, int Vh, unsigned* pmax, Gate gate,
                                cudaStream_t s) {
-  using E = typename K::Store::elem;
-  using G = RtGeom<K, NP, WMODE>;
+  using G = RtGeom<K, NP, MODE>;
   constexpr size_t sm = G::smem;
   constexpr int RT_THREADS = G::threads, RT_WARPS = RT_THREADS / 32;
-  auto kern = k_rows_tc<K, NP, WMODE>;
+  auto kern = k_rows_tc<K, NP, MODE>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 152;
@@ -465,7 +525,8 @@ static cudaError_t launch_rows(void* Q, void* P, void* X, const double2* Sinv, c
   const long long tiles = (3LL * Vh + 15) / 16;
   long long blocks = (tiles + RT_WARPS - 1) / RT_WARPS;
   if (blocks > (long long)sms * G::ctas) blocks = (long long)sms * G::ctas;
-  kern<<<(unsigned)blocks, RT_THREADS, sm, s>>>((E*)Q, (E*)P, (float4*)X, Sinv, BC, SH, N, Vh, pmax,
+  using QE = std::conditional_t<MODE == QROWS, float2, typename K::Store::elem>;
+  kern<<<(unsigned)blocks, RT_THREADS, sm, s>>>((QE*)Q, (typename K::In*)P, (float4*)X, Sinv, BC, SH, N, Vh, pmax,
                                              gate);
   return cudaGetLastError();
 }
@@ -474,13 +535,13 @@ static cudaError_t launch_rows(void* Q, void* P, void* X, const double2* Sinv, c
 // it has run on the tensor cores (error 3.3e-14 of the product's norm); the
 // other widths, which ran in the CUDA cores' double-float (3.1e-15 at N = 3 to
 // 1.1e-14 at N = 32), get the seventh.  FP32: 2.5e-8, the CUDA cores 3.7e-8 to 1.0e-7.
-template <class K, bool WMODE>
+template <class K, int MODE>
 static cudaError_t launch_rows_n(void* Q, void* P, void* X, const double2* Sinv, const double2* BC,
                                  const double2* SH, int N, int Vh, unsigned* pmax, Gate gate,
                                  cudaStream_t s) {
-  if (N <= 8) return launch_rows<K, 8, WMODE>(Q, P, X, Sinv, BC, SH, N, Vh, pmax, gate, s);
-  if (N <= 16) return launch_rows<K, 16, WMODE>(Q, P, X, Sinv, BC, SH, N, Vh, pmax, gate, s);
-  return launch_rows<K, 32, WMODE>(Q, P, X, Sinv, BC, SH, N, Vh, pmax, gate, s);
+  if (N <= 8) return launch_rows<K, 8, MODE>(Q, P, X, Sinv, BC, SH, N, Vh, pmax, gate, s);
+  if (N <= 16) return launch_rows<K, 16, MODE>(Q, P, X, Sinv, BC, SH, N, Vh, pmax, gate, s);
+  return launch_rows<K, 32, MODE>(Q, P, X, Sinv, BC, SH, N, Vh, pmax, gate, s);
 }
 
 cudaError_t bcg_update_rows(FieldKind k, void* Q, void* P, void* X, const double2* Sinv,
@@ -488,9 +549,9 @@ cudaError_t bcg_update_rows(FieldKind k, void* Q, void* P, void* X, const double
                             Gate gate, cudaStream_t s) {
   if (!rows_tc_supported(k, N)) return cudaErrorInvalidValue;
   if (k == FK_F32)
-    return launch_rows_n<KindF32, false>(Q, P, X, Sinv, BC, SH, N, Vh, nullptr, gate, s);
-  if (N == 16) return launch_rows<KindDF, 16, false>(Q, P, X, Sinv, BC, SH, N, Vh, pmax, gate, s);
-  return launch_rows_n<KindDF7, false>(Q, P, X, Sinv, BC, SH, N, Vh, pmax, gate, s);
+    return launch_rows_n<KindF32, UPDATE>(Q, P, X, Sinv, BC, SH, N, Vh, nullptr, gate, s);
+  if (N == 16) return launch_rows<KindDF, 16, UPDATE>(Q, P, X, Sinv, BC, SH, N, Vh, pmax, gate, s);
+  return launch_rows_n<KindDF7, UPDATE>(Q, P, X, Sinv, BC, SH, N, Vh, pmax, gate, s);
 }
 
 cudaError_t w_update_rows(FieldKind k, void* Q, const void* AP, const double2* beta, int N, int Vh,
@@ -498,12 +559,42 @@ cudaError_t w_update_rows(FieldKind k, void* Q, const void* AP, const double2* b
   if (!rows_tc_supported(k, N)) return cudaErrorInvalidValue;
   void* A = const_cast<void*>(AP);
   if (k == FK_F32)
-    return launch_rows_n<KindF32, true>(Q, A, nullptr, beta, nullptr, nullptr, N, Vh, nullptr, gate, s);
+    return launch_rows_n<KindF32, WROWS>(Q, A, nullptr, beta, nullptr, nullptr, N, Vh, nullptr, gate, s);
   if (N == 16)
-    return launch_rows<KindDF, 16, true>(Q, A, nullptr, beta, nullptr, nullptr, N, Vh, nullptr, gate, s);
+    return launch_rows<KindDF, 16, WROWS>(Q, A, nullptr, beta, nullptr, nullptr, N, Vh, nullptr, gate, s);
   if (N == 32)
-    return launch_rows<KindDF, 32, true>(Q, A, nullptr, beta, nullptr, nullptr, N, Vh, nullptr, gate, s);
-  return launch_rows_n<KindDF7, true>(Q, A, nullptr, beta, nullptr, nullptr, N, Vh, nullptr, gate, s);
+    return launch_rows<KindDF, 32, WROWS>(Q, A, nullptr, beta, nullptr, nullptr, N, Vh, nullptr, gate, s);
+  return launch_rows_n<KindDF7, WROWS>(Q, A, nullptr, beta, nullptr, nullptr, N, Vh, nullptr, gate, s);
+}
+
+// Q and P of a reliable update with an FP32 iteration, in two launches (Q is
+// stored in FP32, so reading it back loses nothing): Q = R C^-1 with the 21
+// products of R's double-float slices (error 4e-14, then rounded to FP32), and
+// P = Q + P S with FP32's ten.  On the CUDA cores (k_restart_update) it is bound
+// by the FP64 rate: 24^4, N = 32 (FP64 R) 3477 us, here 362; error of Q 2.5e-8
+// either way, of P 3.6e-8 here and 9.0e-8 (N = 8) to 1.7e-7 (N = 32) there.
+// The line: both launches build their coefficient fragments first, and narrow
+// blocks waste lanes, so small ones stay there (N = 8: V_h = 10368 19 us against
+// 20 here, V_h = 32768 39 against 27; N = 4, V_h = 32768: 15 against 37; N = 16,
+// V_h = 10368: 70 against 30).
+bool restart_rows_supported(FieldKind rk, FieldKind sk, int N, int Vh) {
+  return (rk == FK_F64 || rk == FK_DF) && sk == FK_F32 && N >= 8 && rows_tc_supported(sk, N) &&
+         (long long)Vh * N * N >= 1 << 21;
+}
+
+cudaError_t restart_rows(FieldKind rk, const void* R, void* Q, void* P, const double2* Cinv,
+                         const double2* SH, int init, int N, int Vh, Gate gate, cudaStream_t s) {
+  void* r = const_cast<void*>(R);
+  cudaError_t e =
+      rk == FK_F64
+          ? launch_rows_n<KindF64, QROWS>(Q, r, nullptr, Cinv, nullptr, nullptr, N, Vh, nullptr, gate, s)
+          : launch_rows_n<KindDF, QROWS>(Q, r, nullptr, Cinv, nullptr, nullptr, N, Vh, nullptr, gate, s);
+  if (e != cudaSuccess) return e;
+  if (init)  // P = Q
+    return rk == FK_F64
+               ? launch_rows_n<KindF64, QROWS>(P, r, nullptr, Cinv, nullptr, nullptr, N, Vh, nullptr, gate, s)
+               : launch_rows_n<KindDF, QROWS>(P, r, nullptr, Cinv, nullptr, nullptr, N, Vh, nullptr, gate, s);
+  return launch_rows_n<KindF32, PROWS>(Q, P, nullptr, SH, nullptr, nullptr, N, Vh, nullptr, gate, s);
 }
 
 }  // namespace bcg

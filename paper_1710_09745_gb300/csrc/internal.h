@@ -188,6 +188,10 @@ bool rows_tc_supported(FieldKind k, int N);
 cudaError_t bcg_update_rows(FieldKind k, void* Q, void* P, void* X, const double2* Sinv,
                             const double2* BC, const double2* SH, int N, int Vh, unsigned* pmax,
                             Gate gate, cudaStream_t s);
+// restart_update of the FP32 kind on the tensor cores (large enough blocks)
+bool restart_rows_supported(FieldKind rk, FieldKind sk, int N, int Vh);
+cudaError_t restart_rows(FieldKind rk, const void* R, void* Q, void* P, const double2* Cinv,
+                         const double2* SH, int init, int N, int Vh, Gate gate, cudaStream_t s);
 cudaError_t w_update_rows(FieldKind k, void* Q, const void* AP, const double2* beta, int N, int Vh,
                           Gate gate, cudaStream_t s);
 // the tensor-core fused update (blas_tc.cu): supported (kind, N) pairs

@@ -69,3 +69,24 @@ def test_update_leaves_the_column_maxima(tmp_path, N):
         assert rel.max() <= tol * 1.01, (flags, rel)
         iters.append(info["iters"])
     assert abs(iters[0] - iters[1]) <= 1, iters
+
+
+@pytest.mark.parametrize("dims,N", [((16, 16, 16, 16), 8), ((16, 8, 12, 16), 14),
+                                    ((16, 8, 12, 16), 17), ((12, 8, 8, 16), 31),
+                                    ((12, 8, 8, 16), 32)])
+def test_reliable_updates_of_the_fp32_iteration(dims, N):
+    """Blocks large enough (V_h N^2 >= 2^21) that Q and P of a reliable update come from the
+    tensor cores: the mixed solve meets tol on the oracle's residual, with at most twice the
+    iterations of the double-float form, whose updates are the CUDA cores'."""
+    mass, tol = 0.1, 1e-11
+    b = hi.gaussian_sources(dims, N, seed=51 + N)
+    iters = {}
+    for prec in ("f64", "mixed_f32"):
+        s, fat, lng = gh.make_solver(dims, mass, prec=prec, seed=50, max_rhs=N)
+        X, info = s.solve(b, tol=tol)
+        assert info["status"] == 0 and info["reliable_updates"] >= 1
+        r = (b - hisq.apply_A(dims, fat, lng, mass, gh.to_np(X))).reshape(N, -1)
+        rel = np.linalg.norm(r, axis=1) / np.linalg.norm(b.reshape(N, -1), axis=1)
+        assert rel.max() <= tol * 1.01, (prec, rel)
+        iters[prec] = info["iters"]
+    assert iters["mixed_f32"] <= 2 * iters["f64"], iters
