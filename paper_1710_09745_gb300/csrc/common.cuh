@@ -36,9 +36,10 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // as FP64 adds and format conversions they bound the kernels that convert
 // whole fields (32^4, N = 16: 359 us for a layout conversion whose bytes take
 // 121).  hi is the value rounded to 24 bits, lo the remainder rounded to 24
-// bits, as x - (double)hi gives it; outside 2^-90 .. 2^90, and for zeros, infinities
-// and NaN, the FP64 operations themselves (out of line, or the compiler would
-// execute both sides).
+// bits, as x - (double)hi gives it; outside 2^-90 .. 2^90 (to double: from 2^-72,
+// where a zero or subnormal lo, whose mantissa has no leading one, is still
+// shifted out whole), and for zeros, infinities and NaN, the FP64 operations
+// themselves (out of line, or the compiler would execute both sides).
 __device__ __noinline__ inline df df_from_double_fp64(double x) {
   const float h = __double2float_rn(x);
   return {h, __double2float_rn(x - (double)h)};
@@ -60,7 +61,7 @@ __device__ __noinline__ inline double df_to_double_fp64(df a) { return (double)a
 __device__ __forceinline__ double df_to_double(df a) {
   const unsigned b = __float_as_uint(a.hi), c = __float_as_uint(a.lo);
   const int e = (int)((b >> 23) & 0xff) - 127, le = (int)((c >> 23) & 0xff) - 127;
-  if (e < -90 || e > 90 || le > e - 24) return df_to_double_fp64(a);
+  if (e < -72 || e > 90 || le > e - 24) return df_to_double_fp64(a);
   // lo in units of 2^(e - 52), the result's last place (|lo| <= ulp(hi) / 2)
   const int sh = e - 29 - le;  // >= -5
   const unsigned ml = (c & 0x7fffffu) | 0x800000u;
