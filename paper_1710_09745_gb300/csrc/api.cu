@@ -668,8 +668,8 @@ blockcg_status restart_residual(blockcg_ctx* h, const Ws& w, int N, double tol, 
   TL(TC_GRAM, gram_reduce(w.partials, w.nblocks, N, 1, mat(w, M_G, N), gate, s));
   TL(TC_DENSE, dense_restart(mat(w, M_G, N), mat(w, M_C, N), mat(w, M_CPREV, N), mat(w, M_CINV, N),
                    mat(w, M_SHRU, N), w.bnorm, w.tres, tol, init, cheap ? 0 : 1, N, w.st, gate, ctl, s));
-  TL(TC_STREAM, restart_update(rk, h->sloppy, Rk, w.Q, w.P, mat(w, M_CINV, N), mat(w, M_SHRU, N), init,
-                    N, h->g.Vh, gate, s));
+  TL(TC_STREAM, restart_update(rk, h->sloppy, Rk, mat(w, M_G, N), w.Q, w.P, mat(w, M_CINV, N),
+                    mat(w, M_SHRU, N), init, N, h->g.Vh, gate, s));
   return BLOCKCG_OK;
 }
 

@@ -1094,11 +1094,11 @@ static cudaError_t launch_restart(const void* R, void* Q, void* P, const double2
   return cudaGetLastError();
 }
 
-cudaError_t restart_update(FieldKind rk, FieldKind sk, const void* R, void* Q, void* P,
-                           const double2* Cinv, const double2* SH, int init, int N, int Vh,
-                           Gate gate, cudaStream_t s) {
+cudaError_t restart_update(FieldKind rk, FieldKind sk, const void* R, const double2* G, void* Q,
+                           void* P, const double2* Cinv, const double2* SH, int init, int N,
+                           int Vh, Gate gate, cudaStream_t s) {
   if (restart_rows_supported(rk, sk, N, Vh))
-    return restart_rows(rk, R, Q, P, Cinv, SH, init, N, Vh, gate, s);
+    return restart_rows(rk, R, G, Q, P, Cinv, SH, init, N, Vh, gate, s);
   if (rk == FK_F64 && sk == FK_DF)
     return launch_restart<StoreF64, StoreDF>(R, Q, P, Cinv, SH, init, N, Vh, gate, s);
   if (rk == FK_F64 && sk == FK_F32)

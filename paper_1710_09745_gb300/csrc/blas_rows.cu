@@ -110,9 +110,17 @@ struct KindF32 : SliceKind<StoreF32> {  // four slices, 10 products
 enum RowsMode {
   UPDATE,  // Q = W S^-1 (W in Q), X += P (beta C), P = Q + P S^dag
   WROWS,   // Q = Q - P beta
-  QROWS,   // Q = P C, C upper triangular; Q in FP32, P in the kind's In
+  QROWS,   // Q = P C, C upper triangular; Q in FP32, P in the kind's In; BC = P^dag P
   PROWS,   // P = Q + P S
 };
+
+// x 2^e for a result below 2^1023 (smaller than a normal number: zero), on the
+// integer pipe
+__device__ __forceinline__ double times_pow2(double x, int e) {
+  const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+  if (ex == 0x7ff) return x;
+  return ex == 0 || ex + e <= 0 ? 0.0 : __hiloint2double(hi + e * (1 << 20), __double2loint(x));
+}
 
 template <class K, int NP, int MODE>
 struct RtGeom {
@@ -153,6 +161,11 @@ __global__ void __launch_bounds__((RtGeom<K, NP, MODE>::threads), (RtGeom<K, NP,
   uint2* sB = reinterpret_cast<uint2*>(smem_raw);
   __shared__ int sE[3 * NP];  // column exponents: |column| < 2^e
   __shared__ unsigned sM[NP];  // column maxima of the new P
+  // QROWS: exponents of the norms of P's columns.  The columns are multiplied by
+  // 2^-k and the rows of C by 2^k, or a column far shorter than its neighbours
+  // would lose bits to the scale of its rows (norms of 1 to 1e-12 at 16^4, N = 8:
+  // 195 iterations for 154)
+  __shared__ int sK[NP];
   if (gate_closed(gate)) return;
   const bool keepP = gate.st != nullptr && ((const volatile SolverStatus*)gate.st)->ru_pending;
   auto Ms = [&](int m) { return m == 0 ? Sinv : m == 1 ? BC : SH; };
@@ -160,13 +173,23 @@ __global__ void __launch_bounds__((RtGeom<K, NP, MODE>::threads), (RtGeom<K, NP,
     return i < N && j < N && (MODE == WROWS || MODE == PROWS || rt_in_pattern(m, i, j));
   };
   if (threadIdx.x < NP) sM[threadIdx.x] = 0u;
+  if constexpr (MODE == QROWS) {
+    if (threadIdx.x < NP) {
+      const int j = threadIdx.x;
+      const int ex = j < N ? (__double2hiint(BC[j * N + j].x) >> 20) & 0x7ff : 0;
+      constexpr int KMAX = std::is_same<In, double2>::value ? 512 : 100;
+      sK[j] = ex == 0 || ex == 0x7ff ? 0 : min(max((ex - 1023) >> 1, -KMAX), KMAX);
+    }
+    __syncthreads();
+  }
   for (int c = threadIdx.x; c < NM * NP; c += RT_THREADS) {
     const int m = c / NP, j = c - m * NP;
     double mx = 0.0;
     for (int i = 0; i < N; ++i) {
       if (!in_pattern(m, i, j)) continue;
       const double2 v = Ms(m)[i * N + j];
-      mx = fmax(mx, fmax(fabs(v.x), fabs(v.y)));
+      const double a = fmax(fabs(v.x), fabs(v.y));
+      mx = fmax(mx, MODE == QROWS ? ldexp(a, sK[i]) : a);
     }
     int e = 0;
     if (mx > 0.0 && mx < 1e300) frexp(mx, &e);  // mx in [2^(e-1), 2^e)
@@ -189,9 +212,14 @@ __global__ void __launch_bounds__((RtGeom<K, NP, MODE>::threads), (RtGeom<K, NP,
       double re = 0.0, im = 0.0;
       if (in_pattern(m, i0 + q, j)) {
         const double2 v = Ms(m)[(i0 + q) * N + j];
-        const double sc = ldexp(1.0, -sE[m * NP + j]);
-        re = v.x * sc;
-        im = v.y * sc;
+        if constexpr (MODE == QROWS) {
+          re = ldexp(v.x, sK[i0 + q] - sE[j]);
+          im = ldexp(v.y, sK[i0 + q] - sE[j]);
+        } else {
+          const double sc = ldexp(1.0, -sE[m * NP + j]);
+          re = v.x * sc;
+          im = v.y * sc;
+        }
       }
       // rows (re, im) of column (c, re): Re, -Im; of (c, im): Im, Re
       float4 z = StoreDF::from_double2(part ? make_double2(im, re) : make_double2(re, -im));
@@ -255,25 +283,30 @@ __global__ void __launch_bounds__((RtGeom<K, NP, MODE>::threads), (RtGeom<K, NP,
     // a row hold its N entries)
     auto split = [&](const In (&v)[KS][4], uint32_t (&a)[KS][NSL][4], int (&er)[2]) {
       if constexpr (std::is_same<In, double2>::value) {
-        unsigned mx[2] = {0u, 0u};  // high words
-        auto high = [](double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; };
+        int mx[2] = {0, 0};  // high words, columns scaled
+        auto high = [](double x, int k) {
+          const int h = __double2hiint(x) & 0x7fffffff;
+          return h < (1 << 20) ? 0 : h - k * (1 << 20);
+        };
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
-          for (int i = 0; i < 4; ++i) mx[i & 1] = max(mx[i & 1], max(high(v[ks][i].x), high(v[ks][i].y)));
-        double sc[2];
+          for (int i = 0; i < 4; ++i) {
+            const int k = sK[8 * ks + 2 * t + (i >> 1)];
+            mx[i & 1] = max(mx[i & 1], max(high(v[ks][i].x, k), high(v[ks][i].y, k)));
+          }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           mx[h] = max(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
           mx[h] = max(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
-          er[h] = min(max((int)(mx[h] >> 20) - 1022, -1000), 1000);  // |row| < 2^er
-          sc[h] = __hiloint2double((1023 - er[h]) << 20, 0);
+          er[h] = min(max((mx[h] >> 20) - 1022, -1000), 1000);  // |row| < 2^er
         }
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const double2 z = make_double2(v[ks][i].x * sc[i & 1], v[ks][i].y * sc[i & 1]);
+            const int e = -sK[8 * ks + 2 * t + (i >> 1)] - er[i & 1];
+            const double2 z = make_double2(times_pow2(v[ks][i].x, e), times_pow2(v[ks][i].y, e));
             uint32_t w[NSL];
             K::slices(StoreDF::from_double2(z), 1.f, w);
 #pragma unroll
@@ -325,7 +358,7 @@ __global__ void __launch_bounds__((RtGeom<K, NP, MODE>::threads), (RtGeom<K, NP,
     };
     // (re, im) of output (row h, complex column 4 nt + t)
     auto value = [&](const float (&acc)[NU][4], int h, int er, int ej) {
-      if constexpr (MODE == QROWS) {  // the exponents are large and of opposite sign
+      if constexpr (MODE == QROWS) {  // the exponents may be large and of opposite sign
         const int e = min(max(er + ej, -240), 240);
         er = e / 2;
         ej = e - er;
@@ -369,6 +402,16 @@ __global__ void __launch_bounds__((RtGeom<K, NP, MODE>::threads), (RtGeom<K, NP,
       {
         In v[KS][4];
         load(P, v);
+        if constexpr (MODE == QROWS && std::is_same<In, float4>::value) {
+#pragma unroll
+          for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float f = exp2i(-sK[8 * ks + 2 * t + (i >> 1)]);
+              float4& z = v[ks][i];
+              z = make_float4(__fmul_rn(z.x, f), __fmul_rn(z.y, f), __fmul_rn(z.z, f), __fmul_rn(z.w, f));
+            }
+        }
         split(v, a, er);
       }
 #pragma unroll(NP <= 16 ? NT : 1)
@@ -569,8 +612,9 @@ cudaError_t w_update_rows(FieldKind k, void* Q, const void* AP, const double2* b
 
 // Q and P of a reliable update with an FP32 iteration, in two launches (Q is
 // stored in FP32, so reading it back loses nothing): Q = R C^-1 with the 21
-// products of R's double-float slices (error 4e-14, then rounded to FP32), and
-// P = Q + P S with FP32's ten.  On the CUDA cores (k_restart_update) it is bound
+// products of R's double-float slices (error 4e-14, then rounded to FP32; the
+// columns of R brought to norms of 1 to 2 first, sK), and P = Q + P S with
+// FP32's ten.  On the CUDA cores (k_restart_update) it is bound
 // by the FP64 rate: 24^4, N = 32 (FP64 R) 3477 us, here 362; error of Q 2.5e-8
 // either way, of P 3.6e-8 here and 9.0e-8 (N = 8) to 1.7e-7 (N = 32) there.
 // The line: both launches build their coefficient fragments first, and narrow
@@ -582,18 +626,19 @@ bool restart_rows_supported(FieldKind rk, FieldKind sk, int N, int Vh) {
          (long long)Vh * N * N >= 1 << 21;
 }
 
-cudaError_t restart_rows(FieldKind rk, const void* R, void* Q, void* P, const double2* Cinv,
-                         const double2* SH, int init, int N, int Vh, Gate gate, cudaStream_t s) {
+cudaError_t restart_rows(FieldKind rk, const void* R, const double2* G, void* Q, void* P,
+                         const double2* Cinv, const double2* SH, int init, int N, int Vh,
+                         Gate gate, cudaStream_t s) {
   void* r = const_cast<void*>(R);
   cudaError_t e =
       rk == FK_F64
-          ? launch_rows_n<KindF64, QROWS>(Q, r, nullptr, Cinv, nullptr, nullptr, N, Vh, nullptr, gate, s)
-          : launch_rows_n<KindDF, QROWS>(Q, r, nullptr, Cinv, nullptr, nullptr, N, Vh, nullptr, gate, s);
+          ? launch_rows_n<KindF64, QROWS>(Q, r, nullptr, Cinv, G, nullptr, N, Vh, nullptr, gate, s)
+          : launch_rows_n<KindDF, QROWS>(Q, r, nullptr, Cinv, G, nullptr, N, Vh, nullptr, gate, s);
   if (e != cudaSuccess) return e;
   if (init)  // P = Q
     return rk == FK_F64
-               ? launch_rows_n<KindF64, QROWS>(P, r, nullptr, Cinv, nullptr, nullptr, N, Vh, nullptr, gate, s)
-               : launch_rows_n<KindDF, QROWS>(P, r, nullptr, Cinv, nullptr, nullptr, N, Vh, nullptr, gate, s);
+               ? launch_rows_n<KindF64, QROWS>(P, r, nullptr, Cinv, G, nullptr, N, Vh, nullptr, gate, s)
+               : launch_rows_n<KindDF, QROWS>(P, r, nullptr, Cinv, G, nullptr, N, Vh, nullptr, gate, s);
   return launch_rows_n<KindF32, PROWS>(Q, P, nullptr, SH, nullptr, nullptr, N, Vh, nullptr, gate, s);
 }
 

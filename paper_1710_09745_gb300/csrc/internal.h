@@ -188,10 +188,11 @@ bool rows_tc_supported(FieldKind k, int N);
 cudaError_t bcg_update_rows(FieldKind k, void* Q, void* P, void* X, const double2* Sinv,
                             const double2* BC, const double2* SH, int N, int Vh, unsigned* pmax,
                             Gate gate, cudaStream_t s);
-// restart_update of the FP32 kind on the tensor cores (large enough blocks)
+// restart_update of the FP32 kind on the tensor cores (large enough blocks); G = R^dag R
 bool restart_rows_supported(FieldKind rk, FieldKind sk, int N, int Vh);
-cudaError_t restart_rows(FieldKind rk, const void* R, void* Q, void* P, const double2* Cinv,
-                         const double2* SH, int init, int N, int Vh, Gate gate, cudaStream_t s);
+cudaError_t restart_rows(FieldKind rk, const void* R, const double2* G, void* Q, void* P,
+                         const double2* Cinv, const double2* SH, int init, int N, int Vh,
+                         Gate gate, cudaStream_t s);
 cudaError_t w_update_rows(FieldKind k, void* Q, const void* AP, const double2* beta, int N, int Vh,
                           Gate gate, cudaStream_t s);
 // the tensor-core fused update (blas_tc.cu): supported (kind, N) pairs
@@ -206,10 +207,11 @@ cudaError_t gram_partials_tc(FieldKind k, const void* X, const void* Y, int N, i
                              double2* partials, int nblocks, Gate gate, cudaStream_t s);
 cudaError_t w_update_gram_tc(FieldKind k, void* Q, const void* AP, const double2* beta, int N,
                              int Vh, double2* partials, int nblocks, Gate gate, cudaStream_t s);
-// Q <- R Cinv (converted to Q's kind) ; P <- Q + P SH (or P <- Q when init)
-cudaError_t restart_update(FieldKind rk, FieldKind sk, const void* R, void* Q, void* P,
-                           const double2* Cinv, const double2* SH, int init, int N, int Vh,
-                           Gate gate, cudaStream_t s);
+// Q <- R Cinv (converted to Q's kind) ; P <- Q + P SH (or P <- Q when init);
+// G = R^dag R, from which Cinv comes
+cudaError_t restart_update(FieldKind rk, FieldKind sk, const void* R, const double2* G, void* Q,
+                           void* P, const double2* Cinv, const double2* SH, int init, int N,
+                           int Vh, Gate gate, cudaStream_t s);
 // Y (kind yk) += X (kind xk) ; X = 0
 cudaError_t accumulate(FieldKind yk, FieldKind xk, void* Y, void* X, size_t n_elems, Gate gate,
                        cudaStream_t s);
