@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(256)
   for (int i = lane; i < 144; i += 32) m = max(m, Kind<StoreF64>::key(Ls[i]));
   m = __reduce_max_sync(0xffffffffu, m);
   const int e0 = exp_f64(m);
-  const bool ok = e0 >= -90 && e0 <= 90;  // else the whole field goes to fx_plain
+  const bool ok = e0 >= -90 && e0 <= 90;  // else every half is flagged
   const int e = ok ? e0 : 0;
   if (!ok && lane == 0) atomicOr(bad, 1u);
   // ten lanes per row colour c, so that a lane's column sums stay in registers

@@ -33,8 +33,10 @@
 //
 // A block for which one scale per column will not do (a non-finite or huge
 // entry; in FP64 also a site vector more than 2^9 below its column's maximum,
-// which native FP64 would still resolve to 53 bits; links of that sort) is
-// computed by the same kernel in the kind's own arithmetic (fx_plain).
+// which native FP64 would still resolve to 53 bits), or links without a usable
+// scale, set a flag: the kernel then computes the half in the kind's own
+// arithmetic (fx_cores).  The second half of an operator follows the first one
+// there without looking at its input.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -45,7 +47,7 @@ namespace fx {
 
 // control words in the workspace (Geom::fx_ctl): column maxima of the even
 // and the odd input (bit patterns of |hi|, or the high words of |v| in FP64)
-// and the flag of each that sends the half to fx_plain
+// and the flag of each that sends the half to fx_cores
 constexpr int CTL_MAX = 0;     // + 64 * input parity
 constexpr int CTL_FLAG = 128;  // + input parity
 
@@ -227,17 +229,26 @@ __global__ void __launch_bounds__(256)
 
 // the digit records of a block (HBM-bound: one read, one write of 3/4 of it
 // in double-float): thread = (site, 16 m + gq); clears the other parity's
-// control words, which its stencil accumulates into
+// control words, which its stencil accumulates into.  Nothing to do in a half
+// that is flagged already (by the half before it, or by the links).
 template <class S, int R>
 __global__ void __launch_bounds__(256)
     k_fx_digits(const typename S::elem* __restrict__ f, unsigned char* __restrict__ dig, int N,
-                int NP, int Vh, unsigned* ctl, int slot, Gate gate) {
+                int NP, int Vh, unsigned* ctl, const unsigned* __restrict__ bad_links, int slot,
+                Gate gate) {
   using K = Kind<S>;
   using RC = Rec<K::W, R>;
   constexpr int W = K::W;
   if (gate_closed(gate)) return;
   if (blockIdx.x == 0 && threadIdx.x < 65)
     ctl[threadIdx.x < 64 ? CTL_MAX + 64 * (1 - slot) + threadIdx.x : CTL_FLAG + 1 - slot] = 0u;
+  bool flagged = false;
+  if (threadIdx.x == 0) {
+    flagged = *bad_links != 0u;
+    if (flagged && blockIdx.x == 0) ctl[CTL_FLAG + slot] = 1u;
+    flagged = flagged || ((volatile unsigned*)ctl)[CTL_FLAG + slot] != 0u;
+  }
+  if (__syncthreads_or(flagged)) return;
   __shared__ unsigned cm[64];
   if (threadIdx.x < 64) cm[threadIdx.x] = ctl[CTL_MAX + 64 * slot + threadIdx.x];
   __syncthreads();
@@ -302,7 +313,7 @@ __device__ __forceinline__ unsigned fdiv(unsigned n, const FastDiv& f) {
 struct Args {
   const unsigned char* dig;
   Links L;
-  const unsigned* ctl;
+  unsigned* ctl;
   unsigned* omax;  // column maxima of the output (the second half's input), or null
   int slot, N, NP, parity;
   FastDiv fx, fy, fz, fp;  // extents hx, Ly, Lz; NP
@@ -321,63 +332,39 @@ __device__ __forceinline__ void cp16(uint32_t smem, const void* g) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem), "l"(g));
 }
 
-// the kind's own arithmetic, one thread per (site, right-hand side), for the
-// blocks one scale per column cannot represent
+// The CUDA-core stencil on the digit kernel's grid, for the blocks that one
+// scale per column cannot represent.  12 warps an SM instead of the tuned
+// kernel's 16 to 24: double-float makes up for it with four right-hand sides a
+// thread (at two the link loads bind: 32^4, N = 16 5590 us an operator call
+// against 4960; one 7230; the cp.async kernel 4780).  With less than two rounds
+// of such threads, two right-hand sides (16^4, N = 8 247 us against 267), then one.
+// Warps are dealt out over the SMs in turn, so that few rounds end together
+// (16^4, N = 8 267 us against 305 with whole blocks; 12.8.10.14, N = 5 in FP64
+// 103 against 144, where whole blocks left 64 of 152 SMs idle).  FP64 is bound
+// by its rate either way: within 5 % of the tuned kernel.
 template <class S, int EPI>
-__device__ __noinline__ void fx_plain(const typename S::elem* links, const typename S::elem* in,
+__device__ __noinline__ void fx_cores(const typename S::elem* links, const typename S::elem* in,
                                       typename S::elem* out, const typename S::elem* c1,
                                       const typename S::elem* c2, double m2d, const Geom& g,
-                                      int parity, int N, unsigned* omax) {
-  using C = typename S::comp;
-  using real = typename C::real;
-  using acc = typename C::acc;
-  const real m2 = C::from_double(m2d);
-  const long long total = (long long)g.Vh * N;
-  for (long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x; gid < total;
-       gid += (long long)gridDim.x * blockDim.x) {
-    const int site = (int)(gid / N);
-    const int n = (int)(gid - (long long)site * N);
-    int x, y, z, t;
-    site_xyzt(g, site, parity, x, y, z, t);
-    const int lex = x + g.L[0] * (y + g.L[1] * (z + g.L[2] * t));
-    cpx<acc> a[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) a[i] = czero<C>();
-    const typename S::elem* lp = links + link_offset(g, parity, site);
-#pragma unroll 1
-    for (int d = 0; d < 16; ++d) {
-      const int nb = neighbour_cb_s(g, lex, x, y, z, t, d >> 2, hop_k(d & 3));
-      const typename S::elem* ip = in + (long long)nb * N * 3 + n;
-      cpx<real> v[3];
-#pragma unroll
-      for (int b = 0; b < 3; ++b) v[b] = S::load(ip + b * N);
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int b = 0; b < 3; ++b)
-          cmac<C>(a[i], S::load(lp + (d * 9 + i * 3 + b) * LINK_W), v[b]);
+                                      int parity, int N) {
+  const long long first =
+      ((long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+  const long long step = (long long)gridDim.x * THREADS;
+  const int T4 = (N + 3) / 4, T2 = (N + 1) / 2;
+  if constexpr (std::is_same<S, StoreDF>::value) {
+    if (g.Vh * (long long)T4 >= 2 * step) {
+      dslash_outputs<S, 4, 1, EPI, 0>(links, in, out, c1, c2, m2d, g, parity, N, T4, first,
+                                      g.Vh * (long long)T4, step);
+      return;
     }
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const long long oi = ((long long)site * 3 + i) * N + n;
-      if (EPI != EPI_NONE) {
-        C::neg(a[i].re);
-        C::neg(a[i].im);
-        const cpx<real> cc = S::load(c1 + oi);
-        C::mac(a[i].re, m2, cc.re);
-        C::mac(a[i].im, m2, cc.im);
-        if (EPI == EPI_RESIDUAL) {
-          C::neg(a[i].re);
-          C::neg(a[i].im);
-          const cpx<real> bb = S::load(c2 + oi);
-          C::add(a[i].re, bb.re);
-          C::add(a[i].im, bb.im);
-        }
-      }
-      S::store(out + oi, cfin<C>(a[i]));
-      if (omax) atomicMax(omax + n, Kind<S>::key(out[oi]));
+    if (g.Vh * (long long)T2 >= 2 * step) {
+      dslash_outputs<S, 2, 1, EPI, 0>(links, in, out, c1, c2, m2d, g, parity, N, T2, first,
+                                      g.Vh * (long long)T2, step);
+      return;
     }
   }
+  dslash_outputs<S, 1, 1, EPI, 1>(links, in, out, c1, c2, m2d, g, parity, N, N, first,
+                                  g.Vh * (long long)N, step);
 }
 
 // double-float output: sum_u D_u 2^(-8u), normalised.  The leading digits are
@@ -422,8 +409,9 @@ __global__ void __launch_bounds__(THREADS, 1)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (gate_closed(gate)) return;
   const int N = A.N;
-  if (A.ctl[CTL_FLAG + A.slot] | *A.L.bad) {
-    fx_plain<S, EPI>(links, in, out, c1, c2, m2d, g, A.parity, N, A.omax);
+  if (A.ctl[CTL_FLAG + A.slot]) {
+    if (A.omax && blockIdx.x == 0 && threadIdx.x == 0) A.ctl[CTL_FLAG + 1 - A.slot] = 1u;
+    fx_cores<S, EPI>(links, in, out, c1, c2, m2d, g, A.parity, N);
     return;
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -739,7 +727,8 @@ static cudaError_t run_fx(int flags, int epi, const void* links, const void* in,
                                                                   slot, gate);
   }
   k_fx_digits<S, R><<<cap(((long long)g.Vh * NP * 8 + 255) / 256, 8), 256, 0, s>>>(
-      (const E*)in, (unsigned char*)g.fx_dig, N, NP, g.Vh, g.fx_ctl, slot, gate);
+      (const E*)in, (unsigned char*)g.fx_dig, N, NP, g.Vh, g.fx_ctl, links_of(g.fx_links, g).bad,
+      slot, gate);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   Args A;

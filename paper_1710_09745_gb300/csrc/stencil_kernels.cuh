@@ -153,27 +153,20 @@ __device__ __forceinline__ void unscale_raw(cpx<A>& v) {
   }
 }
 
+// one thread's outputs, the (site, slot) pairs first, first + step, .. < end
+// (k_dslash, and the digit stencil's hand-over)
 template <class S, int RV, int V, int EPI, int UNROLL_HOPS, bool RC = false>
-__global__ void __launch_bounds__(BCG_DSLASH_TPB, (PlainBounds<S, RV>::minb))
-    k_dslash(const typename S::elem* __restrict__ links, const typename S::elem* __restrict__ in,
-             typename S::elem* __restrict__ out, const typename S::elem* __restrict__ c1,
-             const typename S::elem* __restrict__ c2, double m2d, Geom g, int parity, int N,
-             int T, long long span, Gate gate) {
+__device__ __forceinline__ void dslash_outputs(
+    const typename S::elem* __restrict__ links, const typename S::elem* __restrict__ in,
+    typename S::elem* __restrict__ out, const typename S::elem* __restrict__ c1,
+    const typename S::elem* __restrict__ c2, double m2d, const Geom& g, int parity, int N, int T,
+    long long first, long long end, long long step) {
   using C = typename S::comp;
   using real = typename C::real;
   using acc = typename C::acc;
-  if (gate_closed(gate)) return;
   const int NS = N / V;
-  const long long total = (long long)g.Vh * T;
   const real m2 = C::from_double(m2d);
-  // span = 0: grid-stride over (site, slot) pairs; span > 0: this block walks
-  // the contiguous range [blockIdx.x * span, (blockIdx.x + 1) * span) in order,
-  // so that the neighbours a block reads in y (and partly z) were loaded by
-  // the same block shortly before and can still be in its SM's L1
-  const long long g0 = span ? (long long)blockIdx.x * span : (long long)blockIdx.x * blockDim.x;
-  const long long gend = span ? min(total, g0 + span) : total;
-  const long long gstep = span ? (long long)blockDim.x : (long long)gridDim.x * blockDim.x;
-  for (long long gid = g0 + threadIdx.x; gid < gend; gid += gstep) {
+  for (long long gid = first; gid < end; gid += step) {
     const int site = (int)(gid / T);
     const int k = (int)(gid - (long long)site * T);
     int x, y, z, t;
@@ -279,6 +272,25 @@ __global__ void __launch_bounds__(BCG_DSLASH_TPB, (PlainBounds<S, RV>::minb))
       }
     }
   }
+}
+
+template <class S, int RV, int V, int EPI, int UNROLL_HOPS, bool RC = false>
+__global__ void __launch_bounds__(BCG_DSLASH_TPB, (PlainBounds<S, RV>::minb))
+    k_dslash(const typename S::elem* __restrict__ links, const typename S::elem* __restrict__ in,
+             typename S::elem* __restrict__ out, const typename S::elem* __restrict__ c1,
+             const typename S::elem* __restrict__ c2, double m2d, Geom g, int parity, int N,
+             int T, long long span, Gate gate) {
+  if (gate_closed(gate)) return;
+  const long long total = (long long)g.Vh * T;
+  // span = 0: grid-stride over (site, slot) pairs; span > 0: this block walks
+  // the contiguous range [blockIdx.x * span, (blockIdx.x + 1) * span) in order,
+  // so that the neighbours a block reads in y (and partly z) were loaded by
+  // the same block shortly before and can still be in its SM's L1
+  const long long g0 = span ? (long long)blockIdx.x * span : (long long)blockIdx.x * blockDim.x;
+  const long long gend = span ? min(total, g0 + span) : total;
+  const long long gstep = span ? (long long)blockDim.x : (long long)gridDim.x * blockDim.x;
+  dslash_outputs<S, RV, V, EPI, UNROLL_HOPS, RC>(links, in, out, c1, c2, m2d, g, parity, N, T,
+                                                 g0 + threadIdx.x, gend, gstep);
 }
 
 // ---------------------------------------------------------------------------
