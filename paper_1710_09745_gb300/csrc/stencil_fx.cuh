@@ -35,8 +35,7 @@
 // entry; in FP64 also a site vector more than 2^9 below its column's maximum,
 // which native FP64 would still resolve to 53 bits), or links without a usable
 // scale, set a flag: the kernel then computes the half in the kind's own
-// arithmetic (fx_cores).  The second half of an operator follows the first one
-// there without looking at its input.
+// arithmetic (fx_cores).
 #pragma once
 #include <cuda_fp16.h>
 
@@ -230,7 +229,7 @@ __global__ void __launch_bounds__(256)
 // the digit records of a block (HBM-bound: one read, one write of 3/4 of it
 // in double-float): thread = (site, 16 m + gq); clears the other parity's
 // control words, which its stencil accumulates into.  Nothing to do in a half
-// that is flagged already (by the half before it, or by the links).
+// that the links flag.
 template <class S, int R>
 __global__ void __launch_bounds__(256)
     k_fx_digits(const typename S::elem* __restrict__ f, unsigned char* __restrict__ dig, int N,
@@ -242,13 +241,10 @@ __global__ void __launch_bounds__(256)
   if (gate_closed(gate)) return;
   if (blockIdx.x == 0 && threadIdx.x < 65)
     ctl[threadIdx.x < 64 ? CTL_MAX + 64 * (1 - slot) + threadIdx.x : CTL_FLAG + 1 - slot] = 0u;
-  bool flagged = false;
-  if (threadIdx.x == 0) {
-    flagged = *bad_links != 0u;
-    if (flagged && blockIdx.x == 0) ctl[CTL_FLAG + slot] = 1u;
-    flagged = flagged || ((volatile unsigned*)ctl)[CTL_FLAG + slot] != 0u;
+  if (*bad_links) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl[CTL_FLAG + slot] = 1u;
+    return;
   }
-  if (__syncthreads_or(flagged)) return;
   __shared__ unsigned cm[64];
   if (threadIdx.x < 64) cm[threadIdx.x] = ctl[CTL_MAX + 64 * slot + threadIdx.x];
   __syncthreads();
@@ -313,7 +309,7 @@ __device__ __forceinline__ unsigned fdiv(unsigned n, const FastDiv& f) {
 struct Args {
   const unsigned char* dig;
   Links L;
-  unsigned* ctl;
+  const unsigned* ctl;
   unsigned* omax;  // column maxima of the output (the second half's input), or null
   int slot, N, NP, parity;
   FastDiv fx, fy, fz, fp;  // extents hx, Ly, Lz; NP
@@ -335,36 +331,52 @@ __device__ __forceinline__ void cp16(uint32_t smem, const void* g) {
 // The CUDA-core stencil on the digit kernel's grid, for the blocks that one
 // scale per column cannot represent.  12 warps an SM instead of the tuned
 // kernel's 16 to 24: double-float makes up for it with four right-hand sides a
-// thread (at two the link loads bind: 32^4, N = 16 5590 us an operator call
-// against 4960; one 7230; the cp.async kernel 4780).  With less than two rounds
-// of such threads, two right-hand sides (16^4, N = 8 247 us against 267), then one.
-// Warps are dealt out over the SMs in turn, so that few rounds end together
-// (16^4, N = 8 267 us against 305 with whole blocks; 12.8.10.14, N = 5 in FP64
-// 103 against 144, where whole blocks left 64 of 152 SMs idle).  FP64 is bound
-// by its rate either way: within 5 % of the tuned kernel.
+// thread (at two the link loads bind: a half at 32^4, N = 16, with the layout
+// conversions, 3080 us against 2660; one 3820; the cp.async kernel 2530).  With
+// less than two rounds of such threads, two right-hand sides (16^4, N = 8 137 us
+// against 147), then one.  Warps are dealt out over the SMs in turn, so that few
+// rounds end together (16^4, N = 8 147 us against 167 with whole blocks;
+// 12.8.10.14, N = 5 in FP64 60 against 80, where whole blocks left 64 of 152 SMs
+// idle).  FP64 is bound by its rate either way: within 5 % of the tuned kernel.
+// A flagged operator call, both halves: 32^4, N = 16 5150 us (cp.async 4780),
+// N = 8 2660 (2520); 16^4, N = 8 262 (190).
 template <class S, int EPI>
 __device__ __noinline__ void fx_cores(const typename S::elem* links, const typename S::elem* in,
                                       typename S::elem* out, const typename S::elem* c1,
                                       const typename S::elem* c2, double m2d, const Geom& g,
-                                      int parity, int N) {
+                                      int parity, int N, unsigned* smax, unsigned* omax) {
   const long long first =
       ((long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
   const long long step = (long long)gridDim.x * THREADS;
-  const int T4 = (N + 3) / 4, T2 = (N + 1) / 2;
-  if constexpr (std::is_same<S, StoreDF>::value) {
-    if (g.Vh * (long long)T4 >= 2 * step) {
-      dslash_outputs<S, 4, 1, EPI, 0>(links, in, out, c1, c2, m2d, g, parity, N, T4, first,
-                                      g.Vh * (long long)T4, step);
-      return;
+  // the output's column maxima, for the second half (smax: 64 words shared)
+  auto seen = [=](int n, const auto& v) {
+    if (EPI == EPI_NONE && omax) {
+      if constexpr (std::is_same<S, StoreDF>::value)
+        atomicMax(smax + n, Kind<S>::key(make_float4(v.re.hi, v.im.hi, 0.f, 0.f)));
+      else
+        atomicMax(smax + n, Kind<S>::key(make_double2(v.re, v.im)));
     }
-    if (g.Vh * (long long)T2 >= 2 * step) {
-      dslash_outputs<S, 2, 1, EPI, 0>(links, in, out, c1, c2, m2d, g, parity, N, T2, first,
-                                      g.Vh * (long long)T2, step);
-      return;
-    }
+  };
+  if (threadIdx.x < 64) smax[threadIdx.x] = 0u;
+  __syncthreads();
+  auto run = [&](auto r, auto unroll) {
+    constexpr int RV = decltype(r)::value, U = decltype(unroll)::value;
+    const int T = (N + RV - 1) / RV;
+    dslash_outputs<S, RV, 1, EPI, U>(links, in, out, c1, c2, m2d, g, parity, N, T, first,
+                                     g.Vh * (long long)T, step, seen);
+  };
+  using std::integral_constant;
+  constexpr bool DF = std::is_same<S, StoreDF>::value;
+  if (DF && g.Vh * (long long)((N + 3) / 4) >= 2 * step)
+    run(integral_constant<int, DF ? 4 : 1>(), integral_constant<int, DF ? 0 : 1>());
+  else if (DF && g.Vh * (long long)((N + 1) / 2) >= 2 * step)
+    run(integral_constant<int, DF ? 2 : 1>(), integral_constant<int, DF ? 0 : 1>());
+  else
+    run(integral_constant<int, 1>(), integral_constant<int, 1>());
+  if (EPI == EPI_NONE && omax) {
+    __syncthreads();
+    if (threadIdx.x < N && smax[threadIdx.x]) atomicMax(omax + threadIdx.x, smax[threadIdx.x]);
   }
-  dslash_outputs<S, 1, 1, EPI, 1>(links, in, out, c1, c2, m2d, g, parity, N, N, first,
-                                  g.Vh * (long long)N, step);
 }
 
 // double-float output: sum_u D_u 2^(-8u), normalised.  The leading digits are
@@ -410,8 +422,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (gate_closed(gate)) return;
   const int N = A.N;
   if (A.ctl[CTL_FLAG + A.slot]) {
-    if (A.omax && blockIdx.x == 0 && threadIdx.x == 0) A.ctl[CTL_FLAG + 1 - A.slot] = 1u;
-    fx_cores<S, EPI>(links, in, out, c1, c2, m2d, g, A.parity, N);
+    fx_cores<S, EPI>(links, in, out, c1, c2, m2d, g, A.parity, N, (unsigned*)smem_raw, A.omax);
     return;
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

@@ -154,13 +154,18 @@ __device__ __forceinline__ void unscale_raw(cpx<A>& v) {
 }
 
 // one thread's outputs, the (site, slot) pairs first, first + step, .. < end
-// (k_dslash, and the digit stencil's hand-over)
-template <class S, int RV, int V, int EPI, int UNROLL_HOPS, bool RC = false>
+// (k_dslash, and the digit stencil on blocks that digits do not hold); seen(n, v)
+// is called with every output v of right-hand side n
+struct NotSeen {
+  template <class T>
+  __device__ __forceinline__ void operator()(int, const T&) const {}
+};
+template <class S, int RV, int V, int EPI, int UNROLL_HOPS, bool RC = false, class Seen = NotSeen>
 __device__ __forceinline__ void dslash_outputs(
     const typename S::elem* __restrict__ links, const typename S::elem* __restrict__ in,
     typename S::elem* __restrict__ out, const typename S::elem* __restrict__ c1,
     const typename S::elem* __restrict__ c2, double m2d, const Geom& g, int parity, int N, int T,
-    long long first, long long end, long long step) {
+    long long first, long long end, long long step, Seen seen = Seen()) {
   using C = typename S::comp;
   using real = typename C::real;
   using acc = typename C::acc;
@@ -267,7 +272,9 @@ __device__ __forceinline__ void dslash_outputs(
                 C::add(v.im, bb.im);
               }
             }
-            S::store(out + oi, cfin<C>(v));
+            const auto o = cfin<C>(v);
+            S::store(out + oi, o);
+            seen(k * V + w + r * T * V, o);
           }
       }
     }
