@@ -31,11 +31,19 @@
 // Error per term: half a unit of the last digit of either factor, 2^-48
 // (2^-64) of 2^e, and the dropped products s + t >= ND, of that order.
 //
-// A block for which one scale per column will not do (a non-finite or huge
-// entry; in FP64 also a site vector more than 2^9 below its column's maximum,
-// which native FP64 would still resolve to 53 bits), or links without a usable
+// A block for which one scale per column will not do, or links without a usable
 // scale, set a flag: the kernel then computes the half in the kind's own
-// arithmetic (fx_cores).
+// arithmetic (fx_cores).  Will not do: a non-finite or huge entry; in FP64 a
+// nonzero site vector more than 2^9 below its column's maximum, which native
+// FP64 would still resolve to 53 bits; in double-float a run of 8 to 32 sites
+// (a step of k_fx_digits) in which a nonzero column stays more than 2^3 below
+// its maximum, so that 45 of the 48 bits are left of each run's largest entry:
+// what double-float sums keep (3.0e-14 of the result here, digits on Gaussian
+// columns 1.9e-14; without the rule a column that falls as e^-2t lost all but
+// 8 digits in its far slices).  In whole solves with Gaussian sources the
+// maxima of the runs stay within a factor of 4 of the column's (4^4 to 16^4,
+// every iteration); with point sources the first fifth of the iterations is
+// flagged, until the sources have spread.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -226,10 +234,16 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x < N) atomicMax(ctl + CTL_MAX + 64 * slot + threadIdx.x, sm[threadIdx.x]);
 }
 
+// a run's maximum v (FP32 bits) more than 2^3 below its column's c, zero aside
+__device__ __forceinline__ bool low(unsigned v, unsigned c) { return v != 0u && v + (3u << 23) < c; }
+
 // the digit records of a block (HBM-bound: one read, one write of 3/4 of it
-// in double-float): thread = (site, 16 m + gq); clears the other parity's
-// control words, which its stencil accumulates into.  Nothing to do in a half
+// in double-float): thread = (site, 16 m + gq), a CTA takes 8, 16 or 32 sites a
+// step; clears the other parity's control words, which its stencil accumulates
+// into.  Nothing to do in a half
 // that the links flag.
+// sites a step: V_h is a multiple of 8 (even extents), so no run is shorter
+__host__ __device__ inline int digit_sites(int NP) { return NP == 1 ? 32 : NP == 2 ? 16 : 8; }
 template <class S, int R>
 __global__ void __launch_bounds__(256)
     k_fx_digits(const typename S::elem* __restrict__ f, unsigned char* __restrict__ dig, int N,
@@ -245,17 +259,27 @@ __global__ void __launch_bounds__(256)
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl[CTL_FLAG + slot] = 1u;
     return;
   }
-  __shared__ unsigned cm[64];
-  if (threadIdx.x < 64) cm[threadIdx.x] = ctl[CTL_MAX + 64 * slot + threadIdx.x];
+  __shared__ unsigned cm[64], run[2][64];  // maxima: of the columns, of a step's sites
+  if (threadIdx.x < 64) {
+    cm[threadIdx.x] = ctl[CTL_MAX + 64 * slot + threadIdx.x];
+    run[0][threadIdx.x] = run[1][threadIdx.x] = 0u;
+  }
   __syncthreads();
   bool bad = false;
-  const long long total = (long long)Vh * NP * 8;
-  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < total;
-       i += (long long)gridDim.x * 256) {
-    const int gq = (int)(i & 7);
-    const long long sm = i >> 3;
-    const long long site = sm / NP;
-    const int m = (int)(sm - site * NP);
+  const int gq = threadIdx.x & 7, ls = (threadIdx.x >> 3) / NP, m = (threadIdx.x >> 3) - ls * NP;
+  const int per = digit_sites(NP);
+  int par = 0;
+  for (long long s0 = (long long)blockIdx.x * per; s0 < Vh;
+       s0 += (long long)gridDim.x * per, par ^= 1) {
+    const long long site = s0 + ls;
+    if (K::ND == 6 && s0 != (long long)blockIdx.x * per) {
+      // the previous step's maxima; its words are used again after the next barrier
+      __syncthreads();
+      if (threadIdx.x < N) bad = bad || low(run[par ^ 1][threadIdx.x], cm[threadIdx.x]);
+      if (threadIdx.x < N) run[par ^ 1][threadIdx.x] = 0u;
+    }
+    if (ls >= per || site >= Vh) continue;
+    const long long sm = site * NP + m;
     uint32_t w[3][RC::WPC];
 #pragma unroll
     for (int j = 0; j < 3; ++j)
@@ -274,8 +298,10 @@ __global__ void __launch_bounds__(256)
           vm = max(vm, K::key(v));
           K::words(v, e, w[j] + r * W);
         }
-        // FP64: a site vector far below its column's maximum would lose bits
-        if (K::ND == 8 && vm != 0u && (vm >> 20) + 9u < (cm[n] >> 20)) bad = true;
+        if constexpr (K::ND == 8)
+          bad = bad || (vm != 0u && (vm >> 20) + 9u < (cm[n] >> 20));
+        else
+          atomicMax(&run[par][n], vm);
       }
     }
 #pragma unroll
@@ -288,6 +314,10 @@ __global__ void __launch_bounds__(256)
       if constexpr (RC::WPC % 4 == 2)
         reinterpret_cast<uint2*>(o + 128)[gq] = make_uint2(w[j][4], w[j][5]);
     }
+  }
+  if constexpr (K::ND == 6) {  // the last step's maxima
+    __syncthreads();
+    if (threadIdx.x < N) bad = bad || low(run[par ^ 1][threadIdx.x], cm[threadIdx.x]);
   }
   if (bad) atomicOr(ctl + CTL_FLAG + slot, 1u);
 }
@@ -737,7 +767,7 @@ static cudaError_t run_fx(int flags, int epi, const void* links, const void* in,
     k_fx_colmax<S><<<cap((rows + rpb - 1) / rpb, 8), 256, 0, s>>>((const E*)in, N, rows, g.fx_ctl,
                                                                   slot, gate);
   }
-  k_fx_digits<S, R><<<cap(((long long)g.Vh * NP * 8 + 255) / 256, 8), 256, 0, s>>>(
+  k_fx_digits<S, R><<<cap((g.Vh + digit_sites(NP) - 1) / digit_sites(NP), 8), 256, 0, s>>>(
       (const E*)in, (unsigned char*)g.fx_dig, N, NP, g.Vh, g.fx_ctl, links_of(g.fx_links, g).bad,
       slot, gate);
   cudaError_t e = cudaGetLastError();

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 import hisq_inputs as hi
+from oracle import hisq
 from tests import gpu_helpers as gh
 
 pytestmark = pytest.mark.gpu
@@ -69,3 +70,20 @@ def test_time_is_close_to_the_cuda_core_kernels(prec):
                 best = min(best, a.elapsed_time(b))
         ms.append(best)
     assert ms[0] <= 1.25 * ms[1], ms
+
+
+@pytest.mark.parametrize("decades", [0.02, 0.25, 2.0])
+@pytest.mark.parametrize("N", [2, 8, 11, 16, 17, 40])
+def test_falling_columns_in_double_float(N, decades):
+    """A column that falls from time slice to time slice (0.3, 4 and 30 decades over the
+    lattice) keeps double-float's accuracy in every slice, as an operator and as a half."""
+    dims, mass = (4, 4, 4, 16), 0.1
+    psi = hi.gaussian_sources(dims, N, seed=36)
+    t = (np.arange(psi.shape[1]) * 2) // (4 * 4 * 4)
+    psi *= (10.0 ** (-decades * t))[None, :, None]
+    s, fat, lng = gh.make_solver(dims, mass, seed=37, max_rhs=N, dslash_variant=FX)
+    for out, ref in ((s.dslash(psi, 1), hisq.dslash(dims, fat, lng, psi, 1)),
+                     (s.apply_MdagM(psi), hisq.apply_A(dims, fat, lng, mass, psi))):
+        out = gh.to_np(out)
+        for k in range(dims[3]):
+            assert gh.rel_err(out[:, t == k], ref[:, t == k]) < gh.TOL["f64"], k
