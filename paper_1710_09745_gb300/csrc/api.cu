@@ -442,14 +442,16 @@ int stencil_R(blockcg_ctx* h, FieldKind k, int N, const void* links, const void*
                    g0, h->stream);
       return e;
     };
-    // one run first (after the first candidate a run that takes more than
-    // twice the best settles it), then three
-    float ms = 0.f;
-    cudaEventRecord(e0, h->stream);
+    // an untimed run first (a process's first launch of a kernel takes longer
+    // than many a run of it), then one (after the first candidate, a run that
+    // takes more than twice the best settles it), then three
     if (run() != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
+    float ms = 0.f;
+    cudaEventRecord(e0, h->stream);
+    run();
     cudaEventRecord(e1, h->stream);
     if (cudaEventSynchronize(e1) != cudaSuccess) continue;
     cudaEventElapsedTime(&ms, e0, e1);
