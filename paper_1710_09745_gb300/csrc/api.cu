@@ -804,7 +804,24 @@ void tune_block(blockcg_ctx* h, const Ws& w, int N) {
   tune_blas(h, w, N);
   stencil_R(h, h->sloppy, N, h->links_sloppy, w.P, w.Ts, w.AP);
   stencil_R(h, h->fine, N, h->links_fine, w.Y, w.Tf, w.R);
-  if (use_cheap_ru(h, N)) stencil_R(h, h->ru, N, h->links_ru, w.Yru, w.Tf, w.Rru);
+  if (use_cheap_ru(h, N)) {
+    // no update has written Yru yet, and what a fresh workspace holds may read as
+    // values that the digit stencil hands to slower arithmetic
+    if (!h->tuned_R.count((int)h->ru * 128 + N))
+      cudaMemsetAsync(w.Yru, 0, (size_t)h->g.Vh * N * 3 * elem_bytes(h->ru), h->stream);
+    stencil_R(h, h->ru, N, h->links_ru, w.Yru, w.Tf, w.Rru);
+  }
+}
+
+// the same ahead of any solve: P and Y are cleared first, as Yru is there
+blockcg_status tune_ahead(blockcg_ctx* h, const Ws& w, int N) {
+  const size_t nel = (size_t)h->g.Vh * N * 3;
+  if (!h->tuned_R.count((int)h->sloppy * 128 + N))
+    CK(cudaMemsetAsync(w.P, 0, nel * elem_bytes(h->sloppy), h->stream));
+  if (!h->tuned_R.count((int)h->fine * 128 + N))
+    CK(cudaMemsetAsync(w.Y, 0, nel * elem_bytes(h->fine), h->stream));
+  tune_block(h, w, N);
+  return BLOCKCG_OK;
 }
 
 // Algorithm 1 set-up: B and X in internal layout, |b_i|, X = 0 (update),
@@ -1622,10 +1639,8 @@ blockcg_status blockcg_tune(blockcg_t h, int n_rhs) {
   if (rc) return rc;
   const int N = n_rhs;
   Ws w = carve(h, N, h->ws);
-  const size_t nel = (size_t)h->g.Vh * N * 3;
-  CK(cudaMemsetAsync(w.P, 0, nel * elem_bytes(h->sloppy), h->stream));
-  CK(cudaMemsetAsync(w.Y, 0, nel * elem_bytes(h->fine), h->stream));
-  tune_block(h, w, N);
+  rc = tune_ahead(h, w, N);
+  if (rc) return rc;
   CK(cudaStreamSynchronize(h->stream));
   return BLOCKCG_OK;
 }
@@ -1727,16 +1742,17 @@ std::string tune_key(const blockcg_ctx* h, FieldKind k, int N) {
 
 // stencil tuning of one problem, reusing the result of any earlier problem
 // with the same lattice, storage kind and N
-void batch_tune(blockcg_batch* b, blockcg_ctx* h, const Ws& w, int N) {
+blockcg_status batch_tune(blockcg_batch* b, blockcg_ctx* h, const Ws& w, int N) {
   const FieldKind kinds[2] = {h->sloppy, h->fine};
   if (!h->p.dslash_variant)
     for (FieldKind k : kinds) {
       auto it = b->tuned.find(tune_key(h, k, N));
       if (it != b->tuned.end()) h->tuned_R[(int)k * 128 + N] = it->second;
     }
-  tune_block(h, w, N);
-  if (!h->p.dslash_variant)
+  const blockcg_status rc = tune_ahead(h, w, N);
+  if (!rc && !h->p.dslash_variant)
     for (FieldKind k : kinds) b->tuned[tune_key(h, k, N)] = h->tuned_R[(int)k * 128 + N];
+  return rc;
 }
 
 // one chunk of iterations of every active problem, each on its stream,
@@ -1926,7 +1942,8 @@ blockcg_status blockcg_batch_solve(blockcg_batch_t b, const void* const* B, void
     blockcg_ctx* h = b->probs[p];
     reset_instrumentation(h);
     BK(cudaStreamWaitEvent(b->streams[p], b->fork_ev, 0));
-    batch_tune(b, h, carve(h, N[p], h->ws), N[p]);
+    const blockcg_status rc = batch_tune(b, h, carve(h, N[p], h->ws), N[p]);
+    if (rc) return pfail(b, p, rc);
   }
   int chunk = 32;
   for (int p = 0; p < n; ++p) {

@@ -49,3 +49,35 @@ def test_first_use_in_a_process(tmp_path):
     subprocess.run([sys.executable, "-c", FRESH, *map(str, paths)], check=True, cwd=root)
     for p in paths:
         assert choices(p)["kind0", "N8"] & TC
+
+
+@pytest.mark.parametrize("fill", [0, 255])
+def test_batch_tunes_on_a_fresh_workspace(tmp_path, fill):
+    """The workspace of a new handle is uninitialised memory; bytes that read as NaN leave
+    the digit stencil the choice that it is at this size (157 us against 187)."""
+    from paper_1710_09745_gb300 import BlockCGBatch
+    dims, N = (16, 16, 16, 16), 8
+    links = hi.random_links(dims, 51)
+    solvers = [gh.make_solver(dims, 0.1, links=links, max_rhs=N)[0] for _ in range(2)]
+    for s in solvers:
+        s.workspace.fill_(fill)
+    solvers[0].set_tune_cache(tmp_path / "t.json")
+    b = hi.gaussian_sources(dims, N, seed=52)
+    _, infos, _ = BlockCGBatch(solvers).solve([b, b], tol=1e-6)
+    assert all(i["status"] == 0 for i in infos)
+    assert choices(tmp_path / "t.json")["kind0", f"N{N}"] & TC
+
+
+@pytest.mark.parametrize("fill", [0, 255])
+def test_double_float_updates_tune_on_a_fresh_workspace(tmp_path, fill):
+    """The same for the double-float residuals of the FP32 form's reliable updates."""
+    torch = gh.torch_mod()
+    dims, N = (16, 16, 16, 64), 16
+    gen = torch.Generator(device="cuda").manual_seed(53)
+    links = 0.3 * torch.randn((2, 4, int(np.prod(dims)), 3, 3), dtype=torch.complex128,
+                              device="cuda", generator=gen)
+    s, _, _ = gh.make_solver(dims, 0.1, prec="mixed_f32", links=links, max_rhs=N)
+    s.workspace.fill_(fill)
+    s.set_tune_cache(tmp_path / "t.json")
+    s.tune(N)
+    assert choices(tmp_path / "t.json")["kind0", f"N{N}"] & TC
