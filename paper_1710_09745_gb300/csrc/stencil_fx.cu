@@ -16,6 +16,7 @@ __global__ void __launch_bounds__(256)
   __shared__ double2 sL[8 * 145];
   __shared__ uint32_t rec[8][(REC_DIG + REC_EXTRA) / 4];
   __shared__ int sums[8][3][8][2];
+  __shared__ unsigned hop[8][16];  // the largest entries of the hop matrices
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int groups = (g.Vh + 7) / 8;
   const int p = blockIdx.x / groups;
@@ -28,17 +29,26 @@ __global__ void __launch_bounds__(256)
     }
   }
   for (int i = threadIdx.x; i < 8 * 48; i += 256) (&sums[0][0][0][0])[i] = 0;
+  if (threadIdx.x < 8 * 16) (&hop[0][0])[threadIdx.x] = 0u;
   __syncthreads();
   const int site = s0 + warp;
   if (site >= g.Vh) return;
   const double2* Ls = sL + warp * 145;
   unsigned m = 0u;
-  for (int i = lane; i < 144; i += 32) m = max(m, Kind<StoreF64>::key(Ls[i]));
+  for (int i = lane; i < 144; i += 32) {
+    const unsigned v = Kind<StoreF64>::key(Ls[i]);
+    atomicMax(&hop[warp][i / 9], v);
+    m = max(m, v);
+  }
   m = __reduce_max_sync(0xffffffffu, m);
   const int e0 = exp_f64(m);
-  const bool ok = e0 >= -90 && e0 <= 90;  // else every half is flagged
+  const bool ok = e0 >= -90 && e0 <= 90;
   const int e = ok ? e0 : 0;
-  if (!ok && lane == 0) atomicOr(bad, 1u);
+  __syncwarp();
+  const unsigned h = hop[warp][lane & 15];
+  auto below = [&](unsigned by) { return !ok || (h != 0u && h + by < m); };
+  if (__any_sync(0xffffffffu, below(9u << 20)) && lane == 0) atomicOr(bad, 1u);
+  if (__any_sync(0xffffffffu, below(13u << 19)) && lane == 0) atomicOr(bad + 1, 1u);  // 1.5 2^6
   // ten lanes per row colour c, so that a lane's column sums stay in registers
   const int c = lane / 10;
   int sum[8][2] = {};

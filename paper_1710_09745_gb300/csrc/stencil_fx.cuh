@@ -31,9 +31,12 @@
 // Error per term: half a unit of the last digit of either factor, 2^-48
 // (2^-64) of 2^e, and the dropped products s + t >= ND, of that order.
 //
-// A block for which one scale per column will not do, or links without a usable
-// scale, set a flag: the kernel then computes the half in the kind's own
-// arithmetic (fx_cores).  Will not do: a non-finite or huge entry; in FP64 a
+// A block for which one scale per column will not do, or links for which one
+// scale per site will not, set a flag: the kernel then computes the half in the
+// kind's own arithmetic (fx_cores).  Links: an entry outside 2^-90 .. 2^90, or a
+// nonzero hop matrix whose largest entry is less than 2^-9 (double-float 1/96) of
+// the site's: a site whose other neighbours are zero has only that matrix to add
+// up (double-float, 1/360: 3.5e-12; HISQ's three-link term is 1/24).  Blocks: a non-finite or huge entry; in FP64 a
 // nonzero site vector more than 2^9 below its column's maximum, which native
 // FP64 would still resolve to 53 bits; in double-float a run of 8 to 32 sites
 // (a step of k_fx_digits) in which a nonzero column stays more than 2^3 below
@@ -71,7 +74,7 @@ constexpr int REC_EXTRA = 6 * 12 * 8;
 
 struct Links {
   const unsigned char *main, *extra;
-  const unsigned* bad;  // nonzero: some link has no usable scale
+  const unsigned* bad;  // [FP64, double-float]: nonzero if the field is marked
 };
 __host__ __device__ inline Links links_of(const void* base, const Geom& g) {
   const unsigned char* p = (const unsigned char*)base;
@@ -768,8 +771,8 @@ static cudaError_t run_fx(int flags, int epi, const void* links, const void* in,
                                                                   slot, gate);
   }
   k_fx_digits<S, R><<<cap((g.Vh + digit_sites(NP) - 1) / digit_sites(NP), 8), 256, 0, s>>>(
-      (const E*)in, (unsigned char*)g.fx_dig, N, NP, g.Vh, g.fx_ctl, links_of(g.fx_links, g).bad,
-      slot, gate);
+      (const E*)in, (unsigned char*)g.fx_dig, N, NP, g.Vh, g.fx_ctl,
+      links_of(g.fx_links, g).bad + (Kind<S>::ND == 6 ? 1 : 0), slot, gate);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   Args A;

@@ -87,3 +87,23 @@ def test_falling_columns_in_double_float(N, decades):
         out = gh.to_np(out)
         for k in range(dims[3]):
             assert gh.rel_err(out[:, t == k], ref[:, t == k]) < gh.TOL["f64"], k
+
+
+@pytest.mark.parametrize("prec", list(CORES))
+@pytest.mark.parametrize("small", [2.0 ** -4, 2.0 ** -30])
+def test_links_of_very_different_size(prec, small):
+    """Long links far below the fat ones, on a block that is zero but in one time slice: the
+    slices that only the long links reach are as exact as the others."""
+    dims, N = (4, 4, 4, 16), 5
+    fat, lng = hi.random_links(dims, 38)
+    lng = lng * small
+    psi = hi.gaussian_sources(dims, N, seed=39)
+    t = (np.arange(psi.shape[1]) * 2) // (4 * 4 * 4)
+    psi[:, t != 5] = 0
+    s, _, _ = gh.make_solver(dims, 0.1, prec=prec, links=(fat, lng), max_rhs=N, dslash_variant=FX)
+    out, ref = gh.to_np(s.dslash(psi, 1)), hisq.dslash(dims, fat, lng, psi, 1)
+    for k in range(dims[3]):
+        if not np.any(ref[:, t == k]):
+            assert not np.any(out[:, t == k]), k
+        else:
+            assert gh.rel_err(out[:, t == k], ref[:, t == k]) < gh.TOL[prec], k
