@@ -613,6 +613,15 @@ blockcg_status check_ready(blockcg_ctx* h, int N) {
   return BLOCKCG_OK;
 }
 
+// Stencils are timed on zeros: the digit stencil hands some inputs to slower
+// arithmetic, and neither the caller's first block nor what a fresh workspace
+// holds shall decide a choice that outlasts the call.
+blockcg_status clear_untuned(blockcg_ctx* h, FieldKind k, int N, void* in) {
+  if (!h->p.dslash_variant && !h->tuned_R.count((int)k * 128 + N))
+    CK(cudaMemsetAsync(in, 0, (size_t)h->g.Vh * N * 3 * elem_bytes(k), h->stream));
+  return BLOCKCG_OK;
+}
+
 FieldKind op_kind(const blockcg_ctx* h) { return h->sloppy; }
 const void* op_links(const blockcg_ctx* h) { return h->links_sloppy; }
 
@@ -797,30 +806,21 @@ blockcg_status check_solve_args(blockcg_ctx* h, const void* B, const void* X, in
   return BLOCKCG_OK;
 }
 
-// autotune the stencils a block solve of width N uses (no-op once cached)
-// (after the set-up: P and Y hold data; AP, Ts, R and Tf are free until the
-// first iteration and the next reliable update rewrite them)
-void tune_block(blockcg_ctx* h, const Ws& w, int N) {
+// autotune the kernels a block solve of width N uses (no-op once cached), ahead
+// of its set-up, when the workspace holds no state
+blockcg_status tune_ahead(blockcg_ctx* h, const Ws& w, int N) {
   tune_blas(h, w, N);
+  blockcg_status rc = clear_untuned(h, h->sloppy, N, w.P);
+  if (rc) return rc;
   stencil_R(h, h->sloppy, N, h->links_sloppy, w.P, w.Ts, w.AP);
+  rc = clear_untuned(h, h->fine, N, w.Y);
+  if (rc) return rc;
   stencil_R(h, h->fine, N, h->links_fine, w.Y, w.Tf, w.R);
   if (use_cheap_ru(h, N)) {
-    // no update has written Yru yet, and what a fresh workspace holds may read as
-    // values that the digit stencil hands to slower arithmetic
-    if (!h->tuned_R.count((int)h->ru * 128 + N))
-      cudaMemsetAsync(w.Yru, 0, (size_t)h->g.Vh * N * 3 * elem_bytes(h->ru), h->stream);
+    rc = clear_untuned(h, h->ru, N, w.Yru);
+    if (rc) return rc;
     stencil_R(h, h->ru, N, h->links_ru, w.Yru, w.Tf, w.Rru);
   }
-}
-
-// the same ahead of any solve: P and Y are cleared first, as Yru is there
-blockcg_status tune_ahead(blockcg_ctx* h, const Ws& w, int N) {
-  const size_t nel = (size_t)h->g.Vh * N * 3;
-  if (!h->tuned_R.count((int)h->sloppy * 128 + N))
-    CK(cudaMemsetAsync(w.P, 0, nel * elem_bytes(h->sloppy), h->stream));
-  if (!h->tuned_R.count((int)h->fine * 128 + N))
-    CK(cudaMemsetAsync(w.Y, 0, nel * elem_bytes(h->fine), h->stream));
-  tune_block(h, w, N);
   return BLOCKCG_OK;
 }
 
@@ -1292,9 +1292,12 @@ blockcg_status blockcg_dslash(blockcg_t h, const void* in, void* out, int n_rhs,
   Ws w = carve(h, n_rhs, h->ws);
   FieldKind k = op_kind(h);
   Gate g0{nullptr, GATE_ALWAYS};
+  rc = clear_untuned(h, k, n_rhs, w.Q);
+  if (rc) return rc;
+  const int R = stencil_R(h, k, n_rhs, op_links(h), w.Q, w.AP);
   CK(to_internal(k, (const double2*)in, w.Q, n_rhs, h->g.Vh, h->stream));
-  CK(dslash(k, stencil_R(h, k, n_rhs, op_links(h), w.Q, w.AP), EPI_NONE, op_links(h), w.Q, w.AP, nullptr, nullptr, 0.0, h->g,
-            out_parity, n_rhs, g0, h->stream));
+  CK(dslash(k, R, EPI_NONE, op_links(h), w.Q, w.AP, nullptr, nullptr, 0.0, h->g, out_parity, n_rhs,
+            g0, h->stream));
   CK(from_internal(k, w.AP, (double2*)out, n_rhs, h->g.Vh, h->stream));
   return BLOCKCG_OK;
 }
@@ -1306,6 +1309,9 @@ blockcg_status blockcg_apply_MdagM(blockcg_t h, const void* in, void* out, int n
   Ws w = carve(h, n_rhs, h->ws);
   FieldKind k = op_kind(h);
   Gate g0{nullptr, GATE_ALWAYS};
+  rc = clear_untuned(h, k, n_rhs, w.P);
+  if (rc) return rc;
+  stencil_R(h, k, n_rhs, op_links(h), w.P, w.Ts, w.AP);
   CK(to_internal(k, (const double2*)in, w.P, n_rhs, h->g.Vh, h->stream));
   rc = apply_A_internal(h, k, op_links(h), w.P, w.Ts, w.AP, n_rhs, g0);
   if (rc) return rc;
@@ -1394,9 +1400,9 @@ blockcg_status blockcg_solve(blockcg_t h, const void* B, void* X, int n_rhs, dou
   CK(ev.create());
   cudaEvent_t e0 = ev.a, e1 = ev.b;
   CK(cudaEventRecord(e0, s));
-  rc = solve_begin(h, w, B, X, N, tol);
+  rc = tune_ahead(h, w, N);
+  if (!rc) rc = solve_begin(h, w, B, X, N, tol);
   if (rc) return rc;
-  tune_block(h, w, N);
   rc = prime_pmax(h, w, N, Gate{nullptr, GATE_ALWAYS});
   if (rc) return rc;
   SolverStatus hs;

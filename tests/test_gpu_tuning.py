@@ -81,3 +81,16 @@ def test_double_float_updates_tune_on_a_fresh_workspace(tmp_path, fill):
     s.set_tune_cache(tmp_path / "t.json")
     s.tune(N)
     assert choices(tmp_path / "t.json")["kind0", f"N{N}"] & TC
+
+
+@pytest.mark.parametrize("call", ["dslash", "apply_MdagM"])
+def test_the_first_block_does_not_decide(tmp_path, call):
+    """A first block that the digit stencil hands to slower arithmetic (an entry of 1e33)
+    leaves later ones the same choice as any other first block."""
+    dims, N = (16, 16, 16, 16), 16
+    s, _, _ = gh.make_solver(dims, 0.1, seed=54, max_rhs=N)
+    s.set_tune_cache(tmp_path / "t.json")
+    psi = hi.gaussian_sources(dims, N, seed=55)
+    psi[0, 7, 2] = 1e33
+    getattr(s, call)(*((psi, 1) if call == "dslash" else (psi,)))
+    assert choices(tmp_path / "t.json")["kind0", f"N{N}"] & TC
