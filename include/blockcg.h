@@ -319,7 +319,8 @@ blockcg_status blockcg_solve_many(blockcg_t h, const void* B, void* X, int m_rhs
 /* Persist this handle's tuning choices (stencil kernel per storage kind and
  * width, block width of blockcg_solve_many) in the text file `path` (a JSON
  * object of "key": integer lines; created if absent, shared by handles and
- * processes that name it; entries are keyed by lattice, kind, width and
+ * processes that name it; entries are keyed by lattice, kind (FP64 also by its
+ * use: the iteration or the reliable updates of another form), width and
  * device name).  NULL or "" turns persistence off.  Choices already in the
  * file are used instead of timing.  Errors: ERR_ARG (null handle). */
 blockcg_status blockcg_set_tune_cache(blockcg_t h, const char* path);

@@ -344,13 +344,6 @@ std::string dims_tag(const blockcg_ctx* h) {
   return buf;
 }
 
-std::string stencil_key(const blockcg_ctx* h, FieldKind k, int N, int rf) {
-  char buf[160];
-  snprintf(buf, sizeof(buf), "stencil/%s/kind%d/N%d/recon%d/%s", dims_tag(h).c_str(), (int)k, N,
-           rf ? 1 : 0, device_tag().c_str());
-  return buf;
-}
-
 // Register tile of the stencil for (kind, N): tuned once per handle by timing
 // every candidate R on the handle's own buffers (the register-tile tuning of
 // Sec. 6.2); in is read, out is scratch.  Falls back to tile_R on any error.
@@ -378,6 +371,20 @@ bool fx_only(const blockcg_ctx* h, FieldKind k, int N) {
   return k == FK_F64 && N >= 4 && fx_allowed(h, k, N);
 }
 
+// what a stencil choice belongs to.  FP64 has other candidates where it is not the
+// iteration's kind (fx_allowed); that entry is one of its own, so that forms
+// sharing a cache file or a batch do not read each other's.
+std::string stencil_key(const blockcg_ctx* h, FieldKind k, int N) {
+  char buf[160];
+  snprintf(buf, sizeof(buf), "stencil/%s/kind%d/N%d/recon%d/%s", dims_tag(h).c_str(), (int)k, N,
+           recon_flag(h, k) ? 1 : 0, k == FK_F64 && h->sloppy != FK_F64 ? "update/" : "");
+  return buf;
+}
+// whether a stored choice can run: not the digit stencil where it is not a candidate
+bool usable_choice(const blockcg_ctx* h, FieldKind k, int N, long long R) {
+  return !(R & DSLASH_TC) || (k != FK_DF && k != FK_F64) || fx_allowed(h, k, N);
+}
+
 // Autotuned stencil choice for (kind, N), cached.  Each candidate is timed
 // over 3 launches of out = D in; with out2 the candidate is timed on the pair
 // the normal operator runs (out = D_oe in, then out2 = m^2 in - D_eo out), so
@@ -392,7 +399,7 @@ int stencil_R(blockcg_ctx* h, FieldKind k, int N, const void* links, const void*
   if (it != h->tuned_R.end()) return it->second;
   {
     long long v = 0;
-    if (cache_get(h, stencil_key(h, k, N, rf), &v)) {
+    if (cache_get(h, stencil_key(h, k, N) + device_tag(), &v) && usable_choice(h, k, N, v)) {
       h->tuned_R[key] = (int)v;
       return (int)v;
     }
@@ -470,7 +477,7 @@ int stencil_R(blockcg_ctx* h, FieldKind k, int N, const void* links, const void*
   cudaEventDestroy(e1);
   cudaGetLastError();
   h->tuned_R[key] = best;
-  cache_put(h, stencil_key(h, k, N, rf), best);
+  cache_put(h, stencil_key(h, k, N) + device_tag(), best);
   return best;
 }
 
@@ -1739,25 +1746,19 @@ void drop_graph(blockcg_batch* b) {
   b->graph_key.clear();
 }
 
-std::string tune_key(const blockcg_ctx* h, FieldKind k, int N) {
-  char buf[96];
-  snprintf(buf, sizeof(buf), "%d.%d.%d.%d/%d/%d", h->dims[0], h->dims[1], h->dims[2], h->dims[3],
-           (int)k, N);
-  return buf;
-}
-
 // stencil tuning of one problem, reusing the result of any earlier problem
-// with the same lattice, storage kind and N
+// with the same lattice, storage kind and N (stencil_key)
 blockcg_status batch_tune(blockcg_batch* b, blockcg_ctx* h, const Ws& w, int N) {
   const FieldKind kinds[2] = {h->sloppy, h->fine};
   if (!h->p.dslash_variant)
     for (FieldKind k : kinds) {
-      auto it = b->tuned.find(tune_key(h, k, N));
-      if (it != b->tuned.end()) h->tuned_R[(int)k * 128 + N] = it->second;
+      auto it = b->tuned.find(stencil_key(h, k, N));
+      if (it != b->tuned.end() && usable_choice(h, k, N, it->second))
+        h->tuned_R[(int)k * 128 + N] = it->second;
     }
   const blockcg_status rc = tune_ahead(h, w, N);
   if (!rc && !h->p.dslash_variant)
-    for (FieldKind k : kinds) b->tuned[tune_key(h, k, N)] = h->tuned_R[(int)k * 128 + N];
+    for (FieldKind k : kinds) b->tuned[stencil_key(h, k, N)] = h->tuned_R[(int)k * 128 + N];
   return rc;
 }
 

@@ -16,12 +16,13 @@ TC = 8192
 
 
 def choices(path):
-    """{(kind, N): value} of the stencil entries of a tuning cache file"""
+    """{(kind, N): value} of the stencil entries of a tuning cache file (kind2u: FP64 in the
+    reliable updates of another form)"""
     out = {}
     for key, v in json.loads(path.read_text()).items():
         f = key.split("/")
         if f[0] == "stencil":
-            out[f[2], f[3]] = v
+            out[f[2] + ("u" if f[5] == "update" else ""), f[3]] = v
     return out
 
 
@@ -94,3 +95,34 @@ def test_the_first_block_does_not_decide(tmp_path, call):
     psi[0, 7, 2] = 1e33
     getattr(s, call)(*((psi, 1) if call == "dslash" else (psi,)))
     assert choices(tmp_path / "t.json")["kind0", f"N{N}"] & TC
+
+
+@pytest.mark.parametrize("first,second", [("f64", "f64_native"), ("f64_native", "mixed_f32")])
+def test_forms_share_a_cache_file(tmp_path, first, second):
+    """FP64's candidates depend on the form (on 8^4 with N = 4 native FP64 runs on digits and
+    the reliable updates of the others do not): each form finds its own choice."""
+    dims, N = (8, 8, 8, 8), 4
+    links = hi.random_links(dims, 56)
+    for prec in (first, second, first):
+        s, _, _ = gh.make_solver(dims, 0.1, prec=prec, links=links, max_rhs=N)
+        s.set_tune_cache(tmp_path / "t.json")
+        s.tune(N)
+        c = choices(tmp_path / "t.json")
+        if prec == "f64_native":
+            assert c["kind2", f"N{N}"] & TC
+        else:
+            assert not c["kind2u", f"N{N}"] & TC
+
+
+@pytest.mark.parametrize("order", [("f64", "f64_native"), ("f64_native", "f64")])
+def test_forms_share_a_batch(order):
+    from paper_1710_09745_gb300 import BlockCGBatch
+    dims, N = (8, 8, 8, 8), 4
+    links = hi.random_links(dims, 57)
+    solvers = [gh.make_solver(dims, 0.1, prec=p, links=links, max_rhs=N)[0] for p in order]
+    b = hi.gaussian_sources(dims, N, seed=58)
+    _, infos, _ = BlockCGBatch(solvers).solve([b, b], tol=1e-8)
+    assert all(i["status"] == 0 for i in infos)
+    native = solvers[order.index("f64_native")]
+    _, info = native.solve(b, tol=1e-8)
+    assert info["stencil_variant"] & TC
