@@ -182,11 +182,18 @@ void blockcg_default_params(blockcg_params* p);
 blockcg_status blockcg_create(blockcg_t* out, const int dims[4], double mass,
                               const blockcg_params* p, void* stream);
 
-/* Bytes of device memory the caller must provide to blockcg_load_gauge. */
+/* Bytes of device memory to provide to blockcg_load_gauge: all copies of the
+ * links, and the least it takes.  Between them lies the digit form of the
+ * tensor-core stencil (2528 bytes a site of the lattice; F64 and F64_NATIVE
+ * always, the mixed forms from 8192 sites on), which only calls with two and
+ * more right-hand sides read; without it their double-float and FP64 stencils
+ * run on the CUDA cores. */
 size_t blockcg_gauge_bytes(blockcg_t h);
+size_t blockcg_gauge_bytes_min(blockcg_t h);
 
 /* Reorder the caller's links (device complex128 [4][V][3][3] each, layout
- * above) into `storage` (device, >= blockcg_gauge_bytes): per output parity
+ * above) into `storage` (device, >= blockcg_gauge_bytes_min; the digit form is
+ * made if storage_bytes >= blockcg_gauge_bytes): per output parity
  * the 16 hop matrices of Eq. 2 with staggered phases, the factor 1/2, the
  * boundary sign and the backward-hop dagger and minus sign folded in, in
  * the storage formats the precision needs.  The caller may free fat/lng once
@@ -200,7 +207,7 @@ blockcg_status blockcg_load_gauge(blockcg_t h, const void* fat, const void* lng,
                                   size_t storage_bytes);
 
 /* Bytes of device workspace needed by any call on this handle with up to
- * n_rhs right-hand sides. */
+ * n_rhs right-hand sides (less once links without the digit form are loaded). */
 size_t blockcg_workspace_bytes(blockcg_t h, int n_rhs);
 
 /* Hand the handle a caller-owned device workspace (>= the size above for the

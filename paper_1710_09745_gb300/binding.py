@@ -24,7 +24,8 @@ STATUS = {
 
 # every symbol declared in include/blockcg.h
 ABI_SYMBOLS = [
-    "blockcg_default_params", "blockcg_create", "blockcg_gauge_bytes", "blockcg_load_gauge",
+    "blockcg_default_params", "blockcg_create", "blockcg_gauge_bytes",
+    "blockcg_gauge_bytes_min", "blockcg_load_gauge",
     "blockcg_workspace_bytes", "blockcg_set_workspace", "blockcg_dslash", "blockcg_apply_MdagM",
     "blockcg_block_cdot", "blockcg_block_caxpy", "blockcg_thin_qr", "blockcg_solve",
     "blockcg_solve_cg", "blockcg_bench_dslash", "blockcg_destroy", "blockcg_status_string",
@@ -91,6 +92,7 @@ def load_library(path: str = LIB_PATH):
         "blockcg_default_params": (None, [ct.POINTER(Params)]),
         "blockcg_create": (I, [ct.POINTER(P), ct.POINTER(I), D, ct.POINTER(Params), P]),
         "blockcg_gauge_bytes": (S, [P]),
+        "blockcg_gauge_bytes_min": (S, [P]),
         "blockcg_load_gauge": (I, [P, P, P, P, S]),
         "blockcg_workspace_bytes": (S, [P, I]),
         "blockcg_set_workspace": (I, [P, P, S]),
@@ -173,8 +175,8 @@ class BlockCG:
         self.h = h
         self.mass = float(mass)
         self.gauge = None
-        self.load_gauge(fat, lng)
         self.max_rhs = int(max_rhs)
+        self.load_gauge(fat, lng)
         wb = L.blockcg_workspace_bytes(h, self.max_rhs)
         if wb == 0:
             raise BlockCGError(1, "max_rhs out of range")
@@ -188,13 +190,26 @@ class BlockCG:
         L = self.lib
         fat = self._dev(fat, (4, self.V, 3, 3))
         lng = self._dev(lng, (4, self.V, 3, 3))
-        nb = L.blockcg_gauge_bytes(self.h)
         if self.gauge is None:
-            self.gauge = torch.empty(nb, dtype=torch.uint8, device=self.device)
+            self.gauge = torch.empty(self._gauge_bytes(), dtype=torch.uint8, device=self.device)
+        nb = self.gauge.numel()
         self._check(L.blockcg_load_gauge(self.h, ct.c_void_p(fat.data_ptr()),
                                          ct.c_void_p(lng.data_ptr()),
                                          ct.c_void_p(self.gauge.data_ptr()), nb))
         self._links_keepalive = (fat, lng)
+
+    def _gauge_bytes(self):
+        """All copies of the links, or those without the digit form where no call reads it
+        (max_rhs = 1) or it would leave no room for the workspace, a block of max_rhs sources
+        and its solution."""
+        torch = _torch()
+        L = self.lib
+        full, least = L.blockcg_gauge_bytes(self.h), L.blockcg_gauge_bytes_min(self.h)
+        block = self.max_rhs * self.Vh * 3 * 16
+        free = torch.cuda.mem_get_info(self.device)[0] + (
+            torch.cuda.memory_reserved(self.device) - torch.cuda.memory_allocated(self.device))
+        need = full + L.blockcg_workspace_bytes(self.h, self.max_rhs) + 2 * block
+        return least if self.max_rhs == 1 or need > free else full
 
     # ---------------------------------------------------------------- utils
     def _check(self, rc, h="self"):

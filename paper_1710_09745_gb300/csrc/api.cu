@@ -98,6 +98,18 @@ inline size_t up(size_t x) { return (x + ALIGN - 1) / ALIGN * ALIGN; }
 
 enum MatId { M_H = 0, M_G, M_C, M_CPREV, M_BETA, M_BC, M_SINV, M_SH, M_CINV, M_SHRU, M_K, M_RINV, M_COUNT };
 
+// Whether the gauge storage may hold the digit stencil's links.  The forms with an
+// FP32 or 16-bit iteration use them in the reliable updates alone, for FP64 from
+// Vh N = 2^18 (fx_allowed), and N is at most 64: a smaller lattice does without
+// their 2.5 KB per site and parity, and its updates keep the CUDA-core kernels.
+bool fx_stored(const blockcg_ctx* h) {
+  return h->sloppy == FK_DF || h->sloppy == FK_F64 || h->g.Vh >= (1 << 18) / 64;
+}
+// ... and does: not with the least storage (blockcg_gauge_bytes_min)
+bool fx_used(const blockcg_ctx* h) {
+  return fx_stored(h) && (!h->gauge_loaded || h->g.fx_links != nullptr);
+}
+
 struct Ws {
   // fine-kind fields (native FP64); Bru, Yru, Rru: copies in the kind of the
   // early reliable updates (alias B, Y, R when that kind is FP64)
@@ -128,7 +140,7 @@ Ws carve(const blockcg_ctx* h, int N, char* base) {
   // first: the digit stencil's control words and input digits, at offsets
   // that do not depend on N (Geom::fx_ctl and fx_dig, set with the workspace)
   take(FX_CTL_BYTES);
-  take(fx_digit_bytes(h->g, N));
+  if (fx_used(h)) take(fx_digit_bytes(h->g, N));
   size_t nel = (size_t)h->g.Vh * N * 3;
   size_t fb = nel * elem_bytes(h->fine), rb = nel * elem_bytes(h->ru),
          sb = nel * elem_bytes(h->sloppy);
@@ -372,12 +384,15 @@ bool fx_only(const blockcg_ctx* h, FieldKind k, int N) {
 }
 
 // what a stencil choice belongs to.  FP64 has other candidates where it is not the
-// iteration's kind (fx_allowed); that entry is one of its own, so that forms
-// sharing a cache file or a batch do not read each other's.
+// iteration's kind (fx_allowed), and both kinds of the digit stencil have without
+// its links; these entries are their own, so that handles sharing a cache file or
+// a batch do not read each other's.
 std::string stencil_key(const blockcg_ctx* h, FieldKind k, int N) {
   char buf[160];
-  snprintf(buf, sizeof(buf), "stencil/%s/kind%d/N%d/recon%d/%s", dims_tag(h).c_str(), (int)k, N,
-           recon_flag(h, k) ? 1 : 0, k == FK_F64 && h->sloppy != FK_F64 ? "update/" : "");
+  const bool cores = (k == FK_DF || k == FK_F64) && fx_width(N) && fx_stored(h) && !fx_used(h);
+  snprintf(buf, sizeof(buf), "stencil/%s/kind%d/N%d/recon%d/%s%s", dims_tag(h).c_str(), (int)k, N,
+           recon_flag(h, k) ? 1 : 0, k == FK_F64 && h->sloppy != FK_F64 ? "update/" : "",
+           cores ? "cores/" : "");
   return buf;
 }
 // whether a stored choice can run: not the digit stencil where it is not a candidate
@@ -1201,34 +1216,31 @@ void blockcg_destroy(blockcg_t h) {
   delete h;
 }
 
-// Whether the gauge storage holds the digit stencil's links.  The forms with an
-// FP32 or 16-bit iteration use them in the reliable updates alone, for FP64 from
-// Vh N = 2^18 (fx_allowed), and N is at most 64: a smaller lattice does without
-// their 2.5 KB per site and parity, and its updates keep the CUDA-core kernels.
-static bool fx_stored(const blockcg_ctx* h) {
-  return h->sloppy == FK_DF || h->sloppy == FK_F64 || h->g.Vh >= (1 << 18) / 64;
-}
-
-size_t blockcg_gauge_bytes(blockcg_t h) {
+size_t blockcg_gauge_bytes_min(blockcg_t h) {
   if (!h) return 0;
   size_t b = up(links_bytes(h->fine, h->g));
   if (h->sloppy != h->fine) b += up(links_bytes(h->sloppy, h->g, h->p.link_recon));
   if (h->ru != h->fine && h->ru != h->sloppy) b += up(links_bytes(h->ru, h->g));
-  if (fx_stored(h)) b += up(fx_links_bytes(h->g));
   if (h->p.link_recon) b += ALIGN;  // scratch of the link check
   return b;
+}
+
+size_t blockcg_gauge_bytes(blockcg_t h) {
+  if (!h) return 0;
+  return blockcg_gauge_bytes_min(h) + (fx_stored(h) ? up(fx_links_bytes(h->g)) : 0);
 }
 
 blockcg_status blockcg_load_gauge(blockcg_t h, const void* fat, const void* lng, void* storage,
                                   size_t storage_bytes) {
   if (!h) return BLOCKCG_ERR_ARG;
   if (!fat || !lng || !storage) return fail(h, BLOCKCG_ERR_ARG, "null pointer");
-  if (storage_bytes < blockcg_gauge_bytes(h)) return fail(h, BLOCKCG_ERR_NOMEM, "gauge storage too small");
+  const size_t least = blockcg_gauge_bytes_min(h);
+  if (storage_bytes < least) return fail(h, BLOCKCG_ERR_NOMEM, "gauge storage too small");
   const int recon = h->p.link_recon;
   if (recon) {
     // two-row storage needs every link to be a real multiple of an SU(3)
     // matrix, one multiple per kind: check on the device and read the scales
-    char* scratch = (char*)storage + blockcg_gauge_bytes(h) - ALIGN;
+    char* scratch = (char*)storage + least - ALIGN;
     double* c = (double*)scratch;
     int* bad = (int*)(scratch + 2 * sizeof(double));
     CK(check_scaled_su3((const double2*)fat, (const double2*)lng, 2LL * h->g.Vh, 1e-10, c, bad,
@@ -1249,7 +1261,8 @@ blockcg_status blockcg_load_gauge(blockcg_t h, const void* fat, const void* lng,
   h->gauge = storage;
   h->gauge_bytes = storage_bytes;
   // [FP64 links][iteration links, if another kind][reliable-update links, if
-  // a third kind][the digit stencil's links, fx_stored]
+  // a third kind][scratch of the link check][the digit stencil's links, if there
+  // is room]
   char* next = (char*)storage + up(links_bytes(h->fine, h->g));
   h->links_fine = storage;
   h->links_sloppy = storage;
@@ -1266,11 +1279,10 @@ blockcg_status blockcg_load_gauge(blockcg_t h, const void* fat, const void* lng,
   if (h->links_ru != h->links_fine && h->links_ru != h->links_sloppy)
     CK(pack_links(h->ru, (const double2*)fat, (const double2*)lng, h->links_ru, h->g,
                   h->p.antiperiodic_t, 0, h->stream));
-  if (h->ru != h->fine && h->ru != h->sloppy) next += up(links_bytes(h->ru, h->g));
   h->g.fx_links = nullptr;
-  if (fx_stored(h)) {
-    CK(fx_pack_links(h->links_fine, next, h->g, h->stream));
-    h->g.fx_links = next;
+  if (fx_stored(h) && storage_bytes >= blockcg_gauge_bytes(h)) {
+    CK(fx_pack_links(h->links_fine, (char*)storage + least, h->g, h->stream));
+    h->g.fx_links = (char*)storage + least;
   }
   h->gauge_loaded = true;
   return BLOCKCG_OK;

@@ -115,6 +115,7 @@ bool dslash_fx_supported(const Geom& g, int N);
 cudaError_t fx_column_max(const void* f, const Geom& g, int N, Gate gate, cudaStream_t s);
 size_t fx_links_bytes(const Geom& g);
 size_t fx_digit_bytes(const Geom& g, int N);
+bool fx_width(int N);
 // the digit stencil's links from the packed FP64 ones
 cudaError_t fx_pack_links(const void* links_f64, void* storage, const Geom& g, cudaStream_t s);
 bool dslash_tc16_supported(int N);
