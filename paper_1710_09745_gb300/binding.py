@@ -176,11 +176,17 @@ class BlockCG:
         self.mass = float(mass)
         self.gauge = None
         self.max_rhs = int(max_rhs)
-        self.load_gauge(fat, lng)
-        wb = L.blockcg_workspace_bytes(h, self.max_rhs)
-        if wb == 0:
-            raise BlockCGError(1, "max_rhs out of range")
-        self.workspace = torch.empty(wb, dtype=torch.uint8, device=self.device)
+        self._digits = self.max_rhs > 1 and self._room()
+        try:
+            self.load_gauge(fat, lng)
+            self.workspace = self._workspace()
+        except torch.cuda.OutOfMemoryError:
+            if not self._digits:
+                raise
+            self._digits, self.gauge = False, None
+            self.load_gauge(fat, lng)
+            self.workspace = self._workspace()
+        wb = self.workspace.numel()
         self._check(L.blockcg_set_workspace(h, ct.c_void_p(self.workspace.data_ptr()), wb))
 
     def load_gauge(self, fat, lng):
@@ -191,25 +197,33 @@ class BlockCG:
         fat = self._dev(fat, (4, self.V, 3, 3))
         lng = self._dev(lng, (4, self.V, 3, 3))
         if self.gauge is None:
-            self.gauge = torch.empty(self._gauge_bytes(), dtype=torch.uint8, device=self.device)
+            nb = (L.blockcg_gauge_bytes if self._digits else L.blockcg_gauge_bytes_min)(self.h)
+            self.gauge = torch.empty(nb, dtype=torch.uint8, device=self.device)
         nb = self.gauge.numel()
         self._check(L.blockcg_load_gauge(self.h, ct.c_void_p(fat.data_ptr()),
                                          ct.c_void_p(lng.data_ptr()),
                                          ct.c_void_p(self.gauge.data_ptr()), nb))
         self._links_keepalive = (fat, lng)
 
-    def _gauge_bytes(self):
-        """All copies of the links, or those without the digit form where no call reads it
-        (max_rhs = 1) or it would leave no room for the workspace, a block of max_rhs sources
-        and its solution."""
+    def _room(self):
+        """Whether the digit form of the links (read by calls with more than one right-hand
+        side) leaves room for the workspace, a block of max_rhs sources and its solution.
+        Below an eighth of the device's memory it is tried without asking (the query takes
+        longer than a small handle's set-up)."""
         torch = _torch()
         L = self.lib
-        full, least = L.blockcg_gauge_bytes(self.h), L.blockcg_gauge_bytes_min(self.h)
-        block = self.max_rhs * self.Vh * 3 * 16
-        free = torch.cuda.mem_get_info(self.device)[0] + (
+        need = (L.blockcg_gauge_bytes(self.h) + L.blockcg_workspace_bytes(self.h, self.max_rhs)
+                + 2 * self.max_rhs * self.Vh * 3 * 16)
+        if need < torch.cuda.get_device_properties(self.device).total_memory // 8:
+            return True
+        return need <= torch.cuda.mem_get_info(self.device)[0] + (
             torch.cuda.memory_reserved(self.device) - torch.cuda.memory_allocated(self.device))
-        need = full + L.blockcg_workspace_bytes(self.h, self.max_rhs) + 2 * block
-        return least if self.max_rhs == 1 or need > free else full
+
+    def _workspace(self):
+        wb = self.lib.blockcg_workspace_bytes(self.h, self.max_rhs)
+        if wb == 0:
+            raise BlockCGError(1, "max_rhs out of range")
+        return _torch().empty(wb, dtype=_torch().uint8, device=self.device)
 
     # ---------------------------------------------------------------- utils
     def _check(self, rc, h="self"):

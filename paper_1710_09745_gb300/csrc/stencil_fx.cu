@@ -16,7 +16,6 @@ __global__ void __launch_bounds__(256)
   __shared__ double2 sL[8 * 145];
   __shared__ uint32_t rec[8][(REC_DIG + REC_EXTRA) / 4];
   __shared__ int sums[8][3][8][2];
-  __shared__ unsigned hop[8][16];  // the largest entries of the hop matrices
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int groups = (g.Vh + 7) / 8;
   const int p = blockIdx.x / groups;
@@ -29,23 +28,17 @@ __global__ void __launch_bounds__(256)
     }
   }
   for (int i = threadIdx.x; i < 8 * 48; i += 256) (&sums[0][0][0][0])[i] = 0;
-  if (threadIdx.x < 8 * 16) (&hop[0][0])[threadIdx.x] = 0u;
   __syncthreads();
   const int site = s0 + warp;
   if (site >= g.Vh) return;
   const double2* Ls = sL + warp * 145;
-  unsigned m = 0u;
-  for (int i = lane; i < 144; i += 32) {
-    const unsigned v = Kind<StoreF64>::key(Ls[i]);
-    atomicMax(&hop[warp][i / 9], v);
-    m = max(m, v);
-  }
-  m = __reduce_max_sync(0xffffffffu, m);
+  unsigned h = 0u;  // the largest entry of hop matrix lane / 2, by two lanes
+  for (int i = lane & 1; i < 9; i += 2) h = max(h, Kind<StoreF64>::key(Ls[(lane >> 1) * 9 + i]));
+  h = max(h, __shfl_xor_sync(0xffffffffu, h, 1));
+  const unsigned m = __reduce_max_sync(0xffffffffu, h);
   const int e0 = exp_f64(m);
   const bool ok = e0 >= -90 && e0 <= 90;
   const int e = ok ? e0 : 0;
-  __syncwarp();
-  const unsigned h = hop[warp][lane & 15];
   auto below = [&](unsigned by) { return !ok || (h != 0u && h + by < m); };
   if (__any_sync(0xffffffffu, below(9u << 20)) && lane == 0) atomicOr(bad, 1u);
   if (__any_sync(0xffffffffu, below(13u << 19)) && lane == 0) atomicOr(bad + 1, 1u);  // 1.5 2^6

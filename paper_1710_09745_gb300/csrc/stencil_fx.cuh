@@ -258,16 +258,17 @@ __global__ void __launch_bounds__(256)
   if (gate_closed(gate)) return;
   if (blockIdx.x == 0 && threadIdx.x < 65)
     ctl[threadIdx.x < 64 ? CTL_MAX + 64 * (1 - slot) + threadIdx.x : CTL_FLAG + 1 - slot] = 0u;
-  if (*bad_links) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctl[CTL_FLAG + slot] = 1u;
-    return;
-  }
+  const unsigned marked = *bad_links;
   __shared__ unsigned cm[64], run[2][64];  // maxima: of the columns, of a step's sites
   if (threadIdx.x < 64) {
     cm[threadIdx.x] = ctl[CTL_MAX + 64 * slot + threadIdx.x];
     run[0][threadIdx.x] = run[1][threadIdx.x] = 0u;
   }
   __syncthreads();
+  if (marked) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl[CTL_FLAG + slot] = 1u;
+    return;
+  }
   bool bad = false;
   const int gq = threadIdx.x & 7, ls = (threadIdx.x >> 3) / NP, m = (threadIdx.x >> 3) - ls * NP;
   const int per = digit_sites(NP);

@@ -14,9 +14,30 @@ pytestmark = pytest.mark.gpu
 DIMS = (8, 8, 8, 16)  # 8192 sites: all forms have the digit form
 
 
-@pytest.mark.parametrize("prec", ["f64", "f64_native", "mixed_f32", "mixed_f16"])
-@pytest.mark.parametrize("variant", [0, 8192 + 1])
-def test_short_of_memory(monkeypatch, prec, variant):
+class Larger:
+    """blockcg_workspace_bytes, the first answer as of a block that fills the device."""
+
+    def __init__(self, lib, total):
+        self.f, self.total = lib.blockcg_workspace_bytes, total
+
+    def __call__(self, h, n):
+        extra, self.total = self.total, 0
+        return self.f(h, n) + extra
+
+
+def out_of_memory_from(empty, limit):
+    def f(*args, **kw):
+        if args and args[0] == limit:
+            raise gh.torch_mod().cuda.OutOfMemoryError("test")
+        return empty(*args, **kw)
+    return f
+
+
+@pytest.mark.parametrize("short,prec,variant", [
+    ("asked", "f64", 0), ("asked", "f64", 8192 + 1), ("asked", "f64_native", 0),
+    ("asked", "f64_native", 8192 + 1), ("asked", "mixed_f32", 0), ("asked", "mixed_f16", 0),
+    ("tried", "f64", 0), ("tried", "mixed_f32", 0)])
+def test_short_of_memory(monkeypatch, short, prec, variant):
     """With no room for it the handle takes 2528 bytes a site less, and a smaller workspace;
     the operator and a solve meet the oracle (the tensor-core stencil asked for by name runs
     the cp.async or plain kernel)."""
@@ -25,10 +46,14 @@ def test_short_of_memory(monkeypatch, prec, variant):
     links = hi.random_links(DIMS, 41)
     args = dict(prec=prec, links=links, max_rhs=N, dslash_variant=variant)
     full, _, _ = gh.make_solver(DIMS, mass, **args)
-    monkeypatch.setattr(torch.cuda, "mem_get_info", lambda device=None: (0, 1 << 38))
-    monkeypatch.setattr(torch.cuda, "memory_reserved", lambda device=None: 0)
-    monkeypatch.setattr(torch.cuda, "memory_allocated", lambda device=None: 0)
+    if short == "asked":  # a large handle asks for the free memory
+        total = torch.cuda.get_device_properties(0).total_memory
+        monkeypatch.setattr(full.lib, "blockcg_workspace_bytes", Larger(full.lib, total))
+        monkeypatch.setattr(torch.cuda, "mem_get_info", lambda device=None: (0, total))
+    else:  # a small one tries
+        monkeypatch.setattr(torch, "empty", out_of_memory_from(torch.empty, full.workspace.numel()))
     s, fat, lng = gh.make_solver(DIMS, mass, **args)
+    monkeypatch.undo()
     V = int(np.prod(DIMS))
     assert 2528 * V <= full.gauge.numel() - s.gauge.numel() <= 2528 * V + 1024
     assert full.workspace.numel() - s.workspace.numel() == 384 * V // 2  # records of 8 columns
