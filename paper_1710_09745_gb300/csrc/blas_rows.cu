@@ -30,10 +30,16 @@
 // HBM at N <= 8.  32^4, double-float, N = 16 (1.6 M rows): update 738 -> 638 us,
 // W 271 -> 257; 16^4, N = 8: update 40 (CUDA cores) -> 30; FP32 at 24^4, N = 32:
 // update 490 (CUDA cores) -> 325, W and Gram 318 (one kernel) -> 130 + 131.
-// Relative error of the updated blocks against 64 bits: double-float 1.4e-15
-// with 28 products (CUDA cores 3.1e-15 at N = 3 to 1.1e-14 at N = 32), 3.3e-14
-// with the 21 that N = 16 always had here; FP32 2.5e-8 (CUDA cores 3.7e-8 to
-// 1.0e-7).  Which form a problem takes is timed by the BLAS tuner: at N = 12 and
+// Relative error of the updated blocks against 64 bits, columns of like norms:
+// double-float 1.4e-15 with 28 products (CUDA cores 3.1e-15 at N = 3 to 1.1e-14
+// at N = 32), 3.3e-14 with the 21 that N = 16 always had here; FP32 2.5e-8 (CUDA
+// cores 3.7e-8 to 1.0e-7).  A row's scale is its largest entry, so a column k
+// times shorter than the longest is held in log2 k fewer bits, where the CUDA
+// cores hold each entry in all of its own.  The norms of the right-hand sides do
+// not enter W and P.  P's columns differ around peaks of the residual: replayed
+// in 64 bits, FP32 solves at 8^4 with m = 0.02 to 0.001 and N = 5 to 32 have
+// ratios up to 90 and P S^dag 5 to 80 times closer than on the CUDA cores; at
+// m = 1e-4 the ratio reaches 530, and the worst iteration is level with them.  Which form a problem takes is timed by the BLAS tuner: at N = 12 and
 // below the fused CUDA-core W + Gram usually stays ahead of two launches.
 #include <type_traits>
 

@@ -1,6 +1,8 @@
 """GPU tests of the halves that the digit stencil computes in the kind's own arithmetic
 because one scale per column will not do: the values are the CUDA-core kernel's, and the
 time is close to that kernel's."""
+import json
+
 import numpy as np
 import pytest
 
@@ -107,3 +109,31 @@ def test_links_of_very_different_size(prec, small):
             assert not np.any(out[:, t == k]), k
         else:
             assert gh.rel_err(out[:, t == k], ref[:, t == k]) < gh.TOL[prec], k
+
+
+@pytest.mark.parametrize("N", [3, 8, 16, 24])
+@pytest.mark.parametrize("tracked", [False, True])
+def test_point_sources_in_a_solve(tmp_path, N, tracked):
+    """The first iterations of a solve from point sources run flagged halves, the later ones
+    digits, with the maxima of P found by the stencil or left by the tensor-core update: the
+    iterations of the cp.async kernel (one more or less), and tol on the oracle's residual."""
+    torch = gh.torch_mod()
+    dims, mass, tol = (8, 8, 8, 12), 0.1, 1e-11
+    vh = int(np.prod(dims)) // 2
+    b = np.zeros((N, vh, 3), dtype=np.complex128)
+    for j in range(N):
+        b[j, (vh // 2 + 37 * j) % vh, j % 3] = 1
+    dev = torch.cuda.get_device_name().replace(" ", "_")
+    iters = []
+    for v in (CORES["f64"], FX):
+        path = tmp_path / f"{v}.json"
+        flags = 8 | (8 << 8) | (8 << 16) | ((1 << 24) if tracked else 0)
+        path.write_text(json.dumps({f"blas/8.8.8.12/kind0/N{N}/{dev}": flags}))
+        s, fat, lng = gh.make_solver(dims, mass, seed=39, max_rhs=N, dslash_variant=v)
+        s.set_tune_cache(path)
+        X, info = s.solve(b, tol=tol)
+        assert info["status"] == 0
+        r = (b - hisq.apply_A(dims, fat, lng, mass, gh.to_np(X))).reshape(N, -1)
+        assert np.linalg.norm(r, axis=1).max() <= tol * 1.01
+        iters.append(info["iters"])
+    assert abs(iters[0] - iters[1]) <= 1, iters
