@@ -75,7 +75,11 @@ typedef enum {
  *  F64         FP64-accurate iterations: P, Q, AP, T, the update X and the
  *              links stored as double-float pairs (two FP32 words per real,
  *              ~48 significant bits) with error-free-transformation
- *              double-float arithmetic on the FP32 pipes.
+ *              double-float arithmetic on the FP32 pipes, or as exact products
+ *              on the tensor cores.  The tensor-core stencil holds a column in
+ *              48 bits below its maximum; where a run of 8 to 32 sites stays more
+ *              than 2^3 below that (localised or decaying blocks) the half is
+ *              computed on the FP32 pipes instead, to 48 bits of each value.
  *  F64_NATIVE  native FP64 storage and arithmetic in the iterations too (slow
  *              on GPUs with a reduced FP64 rate; for verification).
  *  MIXED_F32   sloppy P, Q, AP, T and links in FP32 with FP32 arithmetic; X

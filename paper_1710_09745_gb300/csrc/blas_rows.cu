@@ -621,7 +621,7 @@ cudaError_t w_update_rows(FieldKind k, void* Q, const void* AP, const double2* b
 // products of R's double-float slices (error 4e-14, then rounded to FP32; the
 // columns of R brought to norms of 1 to 2 first, sK), and P = Q + P S with
 // FP32's ten.  On the CUDA cores (k_restart_update) it is bound
-// by the FP64 rate: 24^4, N = 32 (FP64 R) 3477 us, here 362; error of Q 2.5e-8
+// by the FP64 rate: 24^4, N = 32 (FP64 R) 3477 us, here 385; error of Q 2.5e-8
 // either way, of P 3.6e-8 here and 9.0e-8 (N = 8) to 1.7e-7 (N = 32) there.
 // The line: both launches build their coefficient fragments first, and narrow
 // blocks waste lanes, so small ones stay there (N = 8: V_h = 10368 19 us against
