@@ -127,6 +127,7 @@ typedef struct {
                           grid of contiguous site ranges, 8192 for the
                           tensor-core stencil (mma.sync): double-float and
                           FP64 as exact products of 8-bit digits (N >= 2 with
+                          the digit form of the links, blockcg_gauge_bytes, and
                           a workspace set; the cp.async or the plain kernel
                           otherwise), in the FP16 and
                           bfloat16 forms the stored values themselves (N = 16
